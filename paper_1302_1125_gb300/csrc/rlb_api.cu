@@ -25,6 +25,7 @@ struct rlb_ctx {
     int device;
     int N;
     long long ps;      // plane stride (elements)
+    rlb::Layout lay;   // storage of the populations
     int dim;           // 1, 2 or 3: number of leading axes that are streamed
     int fp32;
     size_t esize;
@@ -229,7 +230,7 @@ rlb_status check_device_status(rlb_ctx *ctx, rlb_status if_bad)
 rlb_status refresh_mirrors(rlb_ctx *ctx)
 {
     if (!ctx->sp.sym || !ctx->sym_stale) return RLB_OK;
-    RLB_CUDA(ctx, rlb::launch_sym(ctx->fp32, 1, ctx->sp.sym, ctx->N, ctx->ps, ctx->fbuf[ctx->cur],
+    RLB_CUDA(ctx, rlb::launch_sym(ctx->fp32, 1, ctx->sp.sym, ctx->N, ctx->lay, ctx->fbuf[ctx->cur],
                                   ctx->hbuf[ctx->cur], ctx->prev, ctx->d_status, ctx->stream));
     ctx->launches += 1;
     ctx->sym_stale = false;
@@ -302,14 +303,38 @@ rlb_status rlb_create(const rlb_grid *grid, int Q, double eta_over_s, double zet
         return cuda_fail(nullptr, e, "cudaGetDevice");
     }
 
+    // bytes of 19 populations and of the previous level: planes, or the FP32
+    // form's blocks of 32 cells with rows padded to even length (the
+    // bulk-staged tiles copy boxes of planes)
+    StepParams &sp = ctx->sp;
+    std::memset(&sp, 0, sizeof(sp));
+    sp.nx = grid->nx;
+    sp.ny = grid->ny;
+    sp.nz = grid->nz;
+    for (int a = 0; a < 3; ++a) {
+        sp.bc_lo[a] = grid->bc_lo[a];
+        sp.bc_hi[a] = grid->bc_hi[a];
+    }
+    sp.lat = o.model;
+    sp.mapping = o.thread_mapping;
+    sp.sym = o.symmetry_1d ? 1 : (o.symmetry_2d ? 2 : 0);
+    const bool bulk = ctx->fp32 && !o.recovery_fp64 && rlb::f32_bulk_eligible(sp, ctx->dim, o.euler_mode);
+    ctx->lay = rlb::Layout{grid->nx, ctx->ps, ctx->fp32 && !bulk};
+    if (ctx->lay.blocked) {
+        const size_t cells = (size_t)(grid->nx + (grid->nx & 1)) * grid->ny * grid->nz;
+        ctx->ps = (long long)align_up(cells, 64);
+    }
+    sp.ps = ctx->ps;
     const size_t plane = (size_t)ctx->ps * ctx->esize;
     const int nb = rlb::totals_blocks(ctx->N);
     size_t off = 0;
     size_t offs[8];
-    offs[0] = off; off += align_up(19 * plane, 256);   // f0
-    offs[1] = off; off += align_up(19 * plane, 256);   // h0
-    offs[2] = off; off += align_up(19 * plane, 256);   // f1
-    offs[3] = off; off += align_up(19 * plane, 256);   // h1
+    // (blocks: f and h of 32 cells interleaved, h starts 19 x 32 values in)
+    const size_t h_at = ctx->lay.blocked ? 19 * 32 * ctx->esize : 19 * plane;
+    offs[0] = off;                                      // f0
+    offs[1] = off + h_at; off += align_up(38 * plane, 256);   // h0
+    offs[2] = off;                                      // f1
+    offs[3] = off + h_at; off += align_up(38 * plane, 256);   // h1
     offs[4] = off; off += align_up(5 * plane, 256);    // prev
     offs[5] = off; off += 256;                          // status
     offs[6] = off; off += align_up(5 * sizeof(double) * nb, 256);   // partial sums
@@ -342,21 +367,8 @@ rlb_status rlb_create(const rlb_grid *grid, int Q, double eta_over_s, double zet
         return cuda_fail(nullptr, e, "cudaMemset");
     }
 
-    StepParams &sp = ctx->sp;
-    std::memset(&sp, 0, sizeof(sp));
-    sp.nx = grid->nx;
-    sp.ny = grid->ny;
-    sp.nz = grid->nz;
-    sp.ps = ctx->ps;
-    for (int a = 0; a < 3; ++a) {
-        sp.bc_lo[a] = grid->bc_lo[a];
-        sp.bc_hi[a] = grid->bc_hi[a];
-    }
     sp.half_lim = limiter == RLB_LIMITER_MINMOD ? 0.5 : 0.0;
-    sp.lat = o.model;
-    sp.mapping = o.thread_mapping;
     sp.slab_by = o.slab_rows > 0 ? o.slab_rows : rlb::f32_slab_rows(grid->nx, grid->ny);
-    sp.sym = o.symmetry_1d ? 1 : (o.symmetry_2d ? 2 : 0);
     sp.k1 = lat_c0ct(o.model) * o.dt_over_dx;
     sp.k2 = double(lat_dmag(o.model)) * lat_c0ct(o.model) * o.dt_over_dx;
     sp.kw = lat_omegaC(o.model) * o.dt_over_dx;
@@ -378,12 +390,18 @@ rlb_status rlb_create(const rlb_grid *grid, int Q, double eta_over_s, double zet
         sp.f_ghost_h[i] = float(sp.ghost_h[i]);
     }
     // the bulk-staged FP32 tiles copy the centre rows and z-neighbour planes
-    // as tensor-map boxes; without the maps the per-thread staged kernel runs
-    if (ctx->fp32 && !o.recovery_fp64 && rlb::f32_bulk_eligible(sp, ctx->dim, o.euler_mode)) {
+    // as tensor-map boxes
+    if (bulk) {
         ctx->have_tmaps = rlb::make_tile_maps(sp, (const float *)ctx->fbuf[0], (const float *)ctx->hbuf[0],
                                               &ctx->tmaps[0]) == cudaSuccess &&
                           rlb::make_tile_maps(sp, (const float *)ctx->fbuf[1], (const float *)ctx->hbuf[1],
                                               &ctx->tmaps[1]) == cudaSuccess;
+        // without the maps the per-thread kernel runs, on blocks (nx is even
+        // and N a multiple of 512: the same sizes)
+        if (!ctx->have_tmaps) {
+            ctx->lay.blocked = 1;
+            for (int k = 0; k < 2; ++k) ctx->hbuf[k] = (char *)ctx->fbuf[k] + 19 * 32 * ctx->esize;
+        }
     }
     ctx->cur = 0;
     ctx->err = "no error";
@@ -411,7 +429,7 @@ rlb_status rlb_init(rlb_ctx *ctx, const double *n, const double *T, const double
             dev[k] = stage + (size_t)k * ctx->N;
         }
     }
-    RLB_CUDA(ctx, rlb::launch_init(ctx->fp32, ctx->N, ctx->ps, dev[0], dev[1], dev[2], dev[3], dev[4],
+    RLB_CUDA(ctx, rlb::launch_init(ctx->fp32, ctx->N, ctx->lay, dev[0], dev[1], dev[2], dev[3], dev[4],
                                    ctx->fbuf[ctx->cur], ctx->hbuf[ctx->cur], ctx->prev, ctx->d_status,
                                    ctx->stream, ctx->sp.lat, ctx->sp.sym));
     ctx->launches += 1;
@@ -429,9 +447,8 @@ rlb_status rlb_step(rlb_ctx *ctx, long long nsteps)
         const int c = ctx->cur, o = 1 - c;
         cudaError_t e;
         if (ctx->fp32 && ctx->opt.recovery_fp64)
-            e = rlb::launch_step_f32_rec64(ctx->sp, ctx->dim, (const float *)ctx->fbuf[c],
-                                           (const float *)ctx->hbuf[c], (float *)ctx->fbuf[o],
-                                           (float *)ctx->hbuf[o], (float *)ctx->prev, ctx->stream);
+            e = rlb::launch_step_f32_rec64(ctx->sp, ctx->dim, (const float *)ctx->fbuf[c], (float *)ctx->fbuf[o],
+                                           (float *)ctx->prev, ctx->stream);
         else if (ctx->fp32)
             e = rlb::launch_step_f32(ctx->sp, ctx->dim, ctx->opt.euler_mode, (const float *)ctx->fbuf[c],
                                      (const float *)ctx->hbuf[c], (float *)ctx->fbuf[o], (float *)ctx->hbuf[o],
@@ -445,7 +462,7 @@ rlb_status rlb_step(rlb_ctx *ctx, long long nsteps)
         ctx->cur = o;
         if (ctx->nsolid > 0) {
             RLB_CUDA(ctx, rlb::launch_solid_reset(ctx->fp32, ctx->nsolid, (const int *)((double *)ctx->solid + 3),
-                                                  ctx->ps, (const double *)ctx->solid, ctx->fbuf[o], ctx->hbuf[o],
+                                                  ctx->lay, (const double *)ctx->solid, ctx->fbuf[o], ctx->hbuf[o],
                                                   ctx->prev, ctx->d_status, ctx->stream, ctx->sp.lat));
             ctx->launches += 1;
         }
@@ -486,7 +503,7 @@ rlb_status rlb_set_solid(rlb_ctx *ctx, const unsigned char *mask, double n, doub
     RLB_CUDA(ctx, cudaMemcpy((double *)ctx->solid + 3, idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice));
     ctx->nsolid = int(idx.size());
     const int c = ctx->cur;
-    RLB_CUDA(ctx, rlb::launch_solid_reset(ctx->fp32, ctx->nsolid, (const int *)((double *)ctx->solid + 3), ctx->ps,
+    RLB_CUDA(ctx, rlb::launch_solid_reset(ctx->fp32, ctx->nsolid, (const int *)((double *)ctx->solid + 3), ctx->lay,
                                           (const double *)ctx->solid, ctx->fbuf[c], ctx->hbuf[c], ctx->prev,
                                           ctx->d_status, ctx->stream, ctx->sp.lat));
     ctx->launches += 1;
@@ -500,7 +517,7 @@ rlb_status rlb_macroscopic(rlb_ctx *ctx, double *out, int on_device)
     RLB_CUDA(ctx, cudaSetDevice(ctx->device));
     if (rlb_status st = refresh_mirrors(ctx); st != RLB_OK) return st;
     double *dst = on_device ? out : (double *)ctx->fbuf[1 - ctx->cur];   // 48 N bytes of staging
-    RLB_CUDA(ctx, rlb::launch_macro(ctx->fp32, ctx->N, ctx->ps, ctx->fbuf[ctx->cur], ctx->hbuf[ctx->cur],
+    RLB_CUDA(ctx, rlb::launch_macro(ctx->fp32, ctx->N, ctx->lay, ctx->fbuf[ctx->cur], ctx->hbuf[ctx->cur],
                                     dst, ctx->d_status, ctx->stream, ctx->sp.lat));
     ctx->launches += 1;
     if (!on_device)
@@ -515,7 +532,7 @@ rlb_status rlb_conserved_totals(rlb_ctx *ctx, double *out)
     if (!out) return fail(ctx, RLB_E_INVALID, "out is NULL");
     RLB_CUDA(ctx, cudaSetDevice(ctx->device));
     if (rlb_status st = refresh_mirrors(ctx); st != RLB_OK) return st;
-    RLB_CUDA(ctx, rlb::launch_totals(ctx->fp32, ctx->N, ctx->ps, ctx->fbuf[ctx->cur], ctx->hbuf[ctx->cur],
+    RLB_CUDA(ctx, rlb::launch_totals(ctx->fp32, ctx->N, ctx->lay, ctx->fbuf[ctx->cur], ctx->hbuf[ctx->cur],
                                      ctx->d_partial, ctx->d_tot, ctx->stream, ctx->sp.lat));
     ctx->launches += 2;
     RLB_CUDA(ctx, cudaMemcpyAsync(ctx->h_tot, ctx->d_tot, 5 * sizeof(double), cudaMemcpyDeviceToHost,
@@ -528,6 +545,28 @@ rlb_status rlb_conserved_totals(rlb_ctx *ctx, double *out)
 size_t rlb_state_bytes(const rlb_ctx *ctx)
 {
     return ctx ? (size_t)43 * ctx->N * ctx->esize : 0;
+}
+
+// the blocks of the FP32 form as compact planes (38 populations, then 5
+// previous-level values) at buf: a device buffer of this GPU directly, any
+// other through the idle population buffer (38 planes of at least N)
+static rlb_status copy_blocks(rlb_ctx *ctx, void *buf, bool out)
+{
+    cudaPointerAttributes at;
+    const bool known = cudaPointerGetAttributes(&at, buf) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    const bool direct = known && at.type == cudaMemoryTypeDevice && at.device == ctx->device && (size_t)buf % 4 == 0;
+    char *user = (char *)buf;
+    for (int k : {38, 5}) {
+        float *blocks = (float *)(k == 38 ? ctx->fbuf[ctx->cur] : ctx->prev);
+        const size_t part = (size_t)k * ctx->N * 4;
+        float *planes = direct ? (float *)user : (float *)ctx->fbuf[1 - ctx->cur];
+        if (!out && !direct) RLB_CUDA(ctx, cudaMemcpyAsync(planes, user, part, cudaMemcpyDefault, ctx->stream));
+        RLB_CUDA(ctx, rlb::launch_state(out, ctx->N, ctx->lay, k, blocks, planes, ctx->stream));
+        if (out && !direct) RLB_CUDA(ctx, cudaMemcpyAsync(user, planes, part, cudaMemcpyDefault, ctx->stream));
+        user += part;
+    }
+    return RLB_OK;
 }
 
 static rlb_status copy_state(rlb_ctx *ctx, void *buf, size_t bytes, bool out)
@@ -544,7 +583,10 @@ static rlb_status copy_state(rlb_ctx *ctx, void *buf, size_t bytes, bool out)
     void *dev[3] = {ctx->fbuf[ctx->cur], ctx->hbuf[ctx->cur], ctx->prev};
     const int rows[3] = {19, 19, 5};
     size_t hoff = 0;
-    for (int k = 0; k < 3; ++k) {
+    if (ctx->lay.blocked) {
+        if (rlb_status st = copy_blocks(ctx, buf, out); st != RLB_OK) return st;
+    }
+    for (int k = 0; k < 3 && !ctx->lay.blocked; ++k) {
         if (out)
             RLB_CUDA(ctx, cudaMemcpy2DAsync(host + hoff, w, dev[k], pitch, w, rows[k], cudaMemcpyDefault,
                                             ctx->stream));
@@ -558,7 +600,7 @@ static rlb_status copy_state(rlb_ctx *ctx, void *buf, size_t bytes, bool out)
         // a reduction steps the class representatives only: every member of
         // a class must equal its representative
         ctx->sym_stale = false;
-        RLB_CUDA(ctx, rlb::launch_sym(ctx->fp32, 0, ctx->sp.sym, ctx->N, ctx->ps, ctx->fbuf[ctx->cur],
+        RLB_CUDA(ctx, rlb::launch_sym(ctx->fp32, 0, ctx->sp.sym, ctx->N, ctx->lay, ctx->fbuf[ctx->cur],
                                       ctx->hbuf[ctx->cur], ctx->prev, ctx->d_status, ctx->stream));
         ctx->launches += 1;
         return check_device_status(ctx, RLB_E_INVALID);

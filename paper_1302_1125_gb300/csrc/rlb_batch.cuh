@@ -47,7 +47,6 @@ __device__ __forceinline__ f32::Geo tube_geo(int off, int nx, int x0)
     g.x0 = x0;
     g.idx0 = off + x0;
     g.has1 = x0 + 1 < nx;
-    g.idx1 = g.has1 ? g.idx0 + 1 : g.idx0;
     g.oa = -2;
     g.oc = 2;
     g.xfix = 0u;
@@ -61,8 +60,6 @@ __device__ __forceinline__ f32::Geo tube_geo(int off, int nx, int x0)
     } else if (x0 + 3 == nx) {
         g.xfix |= f32::XF_HI_ODD3;
     }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) g.yoff[k] = g.zoff[k] = 0;
     return g;
 }
 
@@ -124,9 +121,9 @@ __global__ void __launch_bounds__(MAXT, 1) tubes_kernel(const Args a)
                     // the slots of the shared-memory arrays are MAXT apart (the
                     // launch bound, a compile-time constant: fixed offsets
                     // from one base address), whatever blockDim.x <= MAXT is
-                    f32::update_pair<1, false, true, LD, f32::kParkOn, f32::kStageOn, NP>(
-                        a.p, g, s_eos[i], s_kb[i], f, h, fo, ho, a.prev, a.ps, s_dyn + threadIdx.x, MAXT,
-                        s_dyn + (f32::kParkOn ? f32::kParkSlots * MAXT : 0) + threadIdx.x, MAXT);
+                    f32::StageIO<NP, LD> io{{a.p, f, h, fo, ho, a.prev, a.ps, g.idx0, g.xfix, s_kb[i]},
+                                            g.oa, g.oc, s_dyn + f32::kParkH * MAXT + threadIdx.x, MAXT, 0u};
+                    f32::update_pair<false, false, NP, 0, false>(a.p, io, g.has1, s_eos[i], s_dyn + threadIdx.x, MAXT);
                 }
             }
             if (C > 1) cluster_barrier();
@@ -144,7 +141,7 @@ cudaError_t launch_variant(const Args &a, int threads, int cluster, cudaStream_t
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nclusters_out ? unsigned(cluster) : unsigned(a.nclusters * cluster), 1, 1);
     cfg.blockDim = dim3(unsigned(threads), 1, 1);
-    const size_t smem = f32::step_smem_bytes(MAXT, f32::kStageOn, 1);   // slots MAXT apart
+    const size_t smem = f32::tube_smem_bytes(MAXT);   // slots MAXT apart
     cfg.dynamicSmemBytes = smem;
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));

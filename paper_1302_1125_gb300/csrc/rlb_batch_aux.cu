@@ -28,7 +28,7 @@ __global__ void tubes_init_kernel(const Tube *__restrict__ tubes, const long lon
     if (x0 >= t.nx) return;
     const bool has1 = x0 + 1 < t.nx;
     const long long s0 = pack[b] + x0, d0 = (long long)t.off + x0;
-    const f32::CellPair c{s0, has1 ? s0 + 1 : s0, d0, has1 ? d0 + 1 : d0, has1};
+    const f32::CellPair c{s0, has1 ? s0 + 1 : s0, d0, has1 ? d0 + 1 : d0, has1, d0, has1 ? d0 + 1 : d0};
     f32::init_pair<0, false>(c, ps, n, T, ux, nullptr, nullptr, f, h, prev, status);
 }
 

@@ -47,7 +47,7 @@ namespace rlb {
 namespace f32 {
 
 #ifndef RLB_BULK_BUFS
-#define RLB_BULK_BUFS 6
+#define RLB_BULK_BUFS 5
 #endif
 constexpr int kBulkBufs = RLB_BULK_BUFS;     // items in flight
 constexpr int kRowC = 72;                    // floats per centre row (x0 - 4 .. x0 + 67)
@@ -132,13 +132,13 @@ struct Bulk {
 // stencil values from the tile of one buffer (the Src interface of streamed2)
 struct TileSrc {
     const float *ctr, *zpl;
-    __device__ __forceinline__ f2 get(int slot, int) const
+    __device__ __forceinline__ f2 get(int slot) const
     {
         const float2 v = *reinterpret_cast<const float2 *>(ctr + 2 * (slot - 1));
         return f2{v.x, v.y};
     }
     template <int A, int D>
-    __device__ __forceinline__ f2 nb(int, int) const
+    __device__ __forceinline__ f2 nb(int) const
     {
         static_assert(A == 1 || A == 2, "x neighbours come through get");
         static_assert(D == -2 || D == -1 || D == 1 || D == 2, "distance 1 or 2");
@@ -148,6 +148,7 @@ struct TileSrc {
         const float2 v = *reinterpret_cast<const float2 *>(q);
         return f2{v.x, v.y};
     }
+    __device__ __forceinline__ float extra() const { return 0.0f; }
 };
 
 __device__ __forceinline__ int bulk_map(int c, int n, int lo, int hi)

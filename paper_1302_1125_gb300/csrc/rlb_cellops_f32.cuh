@@ -13,11 +13,42 @@ namespace f32 {
 
 // Two cells: lane 0 reads source index s0 and writes destination index d0,
 // lane 1 the same with s1, d1, written only when has1 (s1 = s0, d1 = d0
-// otherwise).  VEC: d0 and s0 are even, d1 = d0 + 1 and s1 = s0 + 1, so a
-// float plane of even stride moves the pair as one 8-byte access.
+// otherwise); p0, p1 index their previous level.  VEC: the storage indices
+// are even, the second one the first plus 1, so a float plane of even stride
+// moves the pair as one 8-byte access.
 struct CellPair {
     long long s0, s1, d0, d1;
     bool has1;
+    long long p0, p1;
+};
+
+// Storage of a grid's populations (rlb_step_f32.cuh): blocks of 32 cells
+// (blocked = 1; consecutive populations ps = 32 floats apart) or planes of
+// stride ps (the bulk-staged grids, even nx)
+struct Store {
+    int nx, nxe;     // cells of a row, and rounded up to even
+    long long ps;
+    int blocked;
+    // storage index of a grid cell (x fastest)
+    __device__ __forceinline__ long long cell(long long idx) const
+    {
+        if (nx == nxe) return idx;
+        const unsigned row = unsigned(idx) / unsigned(nx);
+        return idx + row;
+    }
+    __device__ __forceinline__ long long at(long long i) const { return blocked ? (long long)blk_at(i) : i; }
+    __device__ __forceinline__ long long prev_at(long long i) const { return blocked ? (long long)blk_prev_at(i) : i; }
+    // the grid cell at an even storage index (the first of a pair)
+    __device__ __forceinline__ long long grid(long long i, bool &has1) const
+    {
+        if (nx == nxe) {
+            has1 = true;
+            return i;
+        }
+        const unsigned row = unsigned(i) / unsigned(nxe);
+        has1 = int(unsigned(i) - row * unsigned(nxe)) + 1 < nx;
+        return i - row;
+    }
 };
 
 template <bool VEC>
@@ -147,11 +178,12 @@ __device__ __forceinline__ void init_pair(const CellPair &c, long long ps, const
         st_cells<VEC>(h + I * ps, c, hv);
         r.template add<I>(fv, hv);
     });
-    st_cells<VEC>(prev + 0 * ps, c, r.S.hi + r.S.lo);
-    st_cells<VEC>(prev + 1 * ps, c, r.Vx.hi + r.Vx.lo);
-    st_cells<VEC>(prev + 2 * ps, c, r.Vy.hi + r.Vy.lo);
-    st_cells<VEC>(prev + 3 * ps, c, r.Vz.hi + r.Vz.lo);
-    st_cells<VEC>(prev + 4 * ps, c, r.H.hi + r.H.lo);
+    const CellPair cp{0, 0, c.p0, c.p1, c.has1, 0, 0};
+    st_cells<VEC>(prev + 0 * ps, cp, r.S.hi + r.S.lo);
+    st_cells<VEC>(prev + 1 * ps, cp, r.Vx.hi + r.Vx.lo);
+    st_cells<VEC>(prev + 2 * ps, cp, r.Vy.hi + r.Vy.lo);
+    st_cells<VEC>(prev + 3 * ps, cp, r.Vz.hi + r.Vz.lo);
+    st_cells<VEC>(prev + 4 * ps, cp, r.H.hi + r.H.lo);
 }
 
 // moments and Landau-frame recovery (Eq. 36, the eigenvalue problem of

@@ -32,6 +32,15 @@ struct StepParams {
     float f_ghost_f[19], f_ghost_h[19];
 };
 
+// Storage of a grid's populations: planes of stride ps (FP64 form; FP32 grids
+// staged by bulk copies), or blocks of 32 cells (the other FP32 grids,
+// rlb_step_f32.cuh)
+struct Layout {
+    int nx;
+    long long ps;
+    int blocked;
+};
+
 // Tensor maps of one buffer of f and h planes (x, y, z, population), with
 // boxes of a tile's centre rows (72 x 12) and of one z-neighbour plane
 // (64 x 8), for the bulk-staged FP32 step
@@ -46,6 +55,7 @@ cudaError_t launch_step_f64(const StepParams &p, int dim, int euler, const doubl
                             double *fo, double *ho, double *prev, cudaStream_t s);
 cudaError_t launch_step_f32(const StepParams &p, int dim, int euler, const float *f, const float *h,
                             float *fo, float *ho, float *prev, cudaStream_t s, const TileMaps *maps = nullptr);
+// (blocked storage: h and ho are not used; with maps: planes)
 // the FP32-storage step on eligible 3-D grids with its stencil tiles staged by
 // bulk copies (rlb_step_f32_bulk.cu); it needs the tensor maps of the buffers
 // it reads (launch_step_f32 runs the per-thread staged kernel without them)
@@ -60,10 +70,10 @@ int f32_slab_rows(int nx, int ny);
 const char *f64_step_kernel_name(const StepParams &p, int dim);
 const char *f32_step_kernel_name(const StepParams &p, int dim, int euler, bool have_maps);
 // the FP32-storage step with the FP64 recovery (rlb_options.recovery_fp64)
-cudaError_t launch_step_f32_rec64(const StepParams &p, int dim, const float *f, const float *h, float *fo,
-                                  float *ho, float *prev, cudaStream_t s);
+cudaError_t launch_step_f32_rec64(const StepParams &p, int dim, const float *f, float *fo, float *prev,
+                                  cudaStream_t s);
 
-cudaError_t launch_init(int fp32, int N, long long ps, const double *n, const double *T,
+cudaError_t launch_init(int fp32, int N, const Layout &l, const double *n, const double *T,
                         const double *ux, const double *uy, const double *uz, void *f, void *h,
                         void *prev, unsigned *status, cudaStream_t s, int lat = 0, int sym = 0);
 // symmetry reductions of grids (sym = 1: 1-D, 2: 2-D; float or double
@@ -71,18 +81,21 @@ cudaError_t launch_init(int fp32, int N, long long ps, const double *n, const do
 // its members' and zeroes the previous level's entries that vanish (the y and
 // z, or the z, components); expand = 0 sets ST_ASYMMETRIC in *status where a
 // member differs from its representative
-cudaError_t launch_sym(int fp32, int expand, int sym, int N, long long ps, void *f, void *h, void *prev,
+cudaError_t launch_sym(int fp32, int expand, int sym, int N, const Layout &l, void *f, void *h, void *prev,
                        unsigned *status, cudaStream_t s);
-cudaError_t launch_macro(int fp32, int N, long long ps, const void *f, const void *h, double *out,
+cudaError_t launch_macro(int fp32, int N, const Layout &l, const void *f, const void *h, double *out,
                          unsigned *status, cudaStream_t s, int lat = 0);
+// FP32 blocks <-> compact planes of N: the 38 populations (k = 38) or the 5
+// previous-level values (k = 5) of every cell
+cudaError_t launch_state(bool out, int N, const Layout &l, int k, float *blocks, float *planes, cudaStream_t s);
 // partial holds 5 * totals_blocks(N) doubles; out 5 doubles (device)
 int totals_blocks(int N);
-cudaError_t launch_totals(int fp32, int N, long long ps, const void *f, const void *h,
+cudaError_t launch_totals(int fp32, int N, const Layout &l, const void *f, const void *h,
                           double *partial, double *out, cudaStream_t s, int lat = 0);
 
 // solid cells: the M cells idx[0..M) are set to the equilibrium of the
 // state st = {n, T, 0} (device doubles) in f, h and the previous level
-cudaError_t launch_solid_reset(int fp32, int M, const int *idx, long long ps, const double *st, void *f,
+cudaError_t launch_solid_reset(int fp32, int M, const int *idx, const Layout &l, const double *st, void *f,
                                void *h, void *prev, unsigned *status, cudaStream_t s, int lat = 0);
 
 // set the text rlb_last_error(NULL) returns on this thread

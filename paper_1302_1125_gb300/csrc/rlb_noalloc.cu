@@ -72,7 +72,7 @@ extern "C" rlb_status rlb_conserved_totals_noalloc(const void *f, const void *h,
     }
     // every partial slot the finishing kernel reads is written earlier in the
     // same call, so nothing has to be cleared between calls
-    const cudaError_t e = rlb::launch_totals(precision == RLB_FP32_STORAGE, N, plane_stride, f, h,
+    const cudaError_t e = rlb::launch_totals(precision == RLB_FP32_STORAGE, N, rlb::Layout{N, plane_stride, 0}, f, h,
                                              partial, out_device, (cudaStream_t)cuda_stream);
     if (e != cudaSuccess) {
         rlb::set_thread_error(cudaGetErrorString(e));

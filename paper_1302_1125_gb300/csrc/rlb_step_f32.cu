@@ -10,8 +10,8 @@ cudaError_t launch_step_f32(const StepParams &p, int dim, int euler, const float
                             float *fo, float *ho, float *prev, cudaStream_t s, const TileMaps *maps)
 {
     if (maps && f32_bulk_eligible(p, dim, euler)) return launch_step_f32_bulk(p, f, h, fo, ho, prev, maps, s);
-    if (f32_use_linear(p, dim)) return launch_step_f32_linear(p, dim, euler, f, h, fo, ho, prev, s);
-    return launch_f32_mapped<false>(p, dim, euler, f, h, fo, ho, prev, s);
+    if (f32_use_linear(p, dim)) return launch_step_f32_linear(p, dim, euler, f, fo, prev, s);
+    return launch_f32_mapped<false>(p, dim, euler, f, fo, prev, s);
 }
 
 // One z-plane of a slab (the f and h planes of its block rows) about this

@@ -55,146 +55,114 @@ using rlb::has_vz;
 using rlb::mult;
 using rlb::rep;
 
-// geometry of one thread's pair of cells
-struct Geo {
-    int idx0, idx1;      // cell indices (idx1 = idx0 when x0 + 1 is outside the grid)
-    int x0;
-    bool has1;
-    int oa, oc;          // offsets of the pairs holding x0-2, x0-1 and x0+2, x0+3
-    unsigned xfix;       // edge columns: clamp or ghost fix-ups (XF_*)
-    int yoff[4], zoff[4];   // offsets of rows/planes at -2, -1, +1, +2 (mapped)
-    // 3-D staged step: byte offsets, from the start of a population plane, of
-    // the pairs a thread stages: x0-2, x0, x0+2 (mapped like oa, oc), then the
-    // rows at y-2, y-1, y+1, y+2 and the planes at z-2 .. z+2 (mapped); 32
-    // bits hold them since FP32 grids have fewer than 2^30 cells
-    unsigned sb[11];
-};
-// XF_HI_ODD1 / XF_HI_ODD3: odd-length tube stored with one pad cell, the pair
-// holds its last cell (x0 = nx - 1) or ends two cells before it (x0 = nx - 3)
-enum { XF_LO_CLAMP = 1, XF_LO_GHOST = 2, XF_HI_CLAMP = 4, XF_HI_GHOST = 8, XF_HI_ODD1 = 16, XF_HI_ODD3 = 32 };
+// Storage of a grid in FP32 form: rows are padded to an even length nxe =
+// nx + nx % 2, and cell (x, y, z) has the storage index i = x + nxe (y + ny z).
+// Blocks of kBlk consecutive storage cells hold their 38 populations (f, then
+// h) one after the other: population k of cell i is at float
+//   (i / kBlk) kBlk 38 + k kBlk + i % kBlk,
+// so that every population of a cell sits at a compile-time distance from its
+// first one and a thread needs one address per stencil position for all 38
+// (with one plane per population each load cost two more instructions for its
+// address, 14 % of the step's instructions).  A pair of cells (even i) never
+// straddles a block; 32 cells are one 128-byte line per population.  The
+// previous level has 5 values per cell in blocks of its own.
+constexpr int kBlk = 32;
+constexpr int kPops = 38;
+__host__ __device__ __forceinline__ size_t blk_at(long long i) { return size_t(i >> 5) * (kBlk * kPops) + size_t(i & 31); }
+__host__ __device__ __forceinline__ size_t blk_prev_at(long long i) { return size_t(i >> 5) * (kBlk * 5) + size_t(i & 31); }
 
-__device__ __forceinline__ int map1(int c, int n, int lo, int hi, bool &ghost)
+// Fix-ups of the x stencil v[0..5] = x0-2 .. x0+3 of a pair at a row's ends:
+// clamped (open) or ghost (inlet) values, and the ends of rows of odd length,
+// whose last pair (ODD1: x0 = nx - 1) holds one pad cell and whose last but
+// one (ODD3: x0 = nx - 3) ends two cells before it.  Periodic rows of even
+// length need none (the pair's address wraps); those of odd length take one
+// extra value (EX) where the wrapped cells are not an aligned pair.
+enum {
+    XF_LO_CLAMP = 1, XF_LO_GHOST = 2, XF_HI_CLAMP = 4, XF_HI_GHOST = 8, XF_HI_ODD1 = 16, XF_HI_ODD3 = 32,
+    XF_HI_ODD1G = 64, XF_HI_ODD3G = 128, XF_LO_EX = 256, XF_HI_EX = 512, XF_HI_WRAP1 = 1024, XF_HI_SELF = 2048
+};
+
+__device__ __forceinline__ int map1(int c, int n, int lo, int hi)
 {
-    ghost = false;
     if (c >= 0 && c < n) return c;
     const int bc = c < 0 ? lo : hi;
     if (bc == BC_PERIODIC) {
         int m = c % n;
         return m < 0 ? m + n : m;
     }
-    if (bc == BC_OUTFLOW) return c < 0 ? 0 : n - 1;
-    ghost = true;
     return c < 0 ? 0 : n - 1;
 }
 
-// Load kinds.  LD_NC: read-only path, for a launch that never writes the
-// populations it reads.  A persistent launch reads what it wrote in earlier
-// steps: LD_CA (cached in L1) when only threads of the same block wrote the
-// data (ordered by the block barrier), LD_CG (cached in L2 only) when other
-// blocks of the cluster wrote it on other SMs.
-enum { LD_NC = 0, LD_CA = 1, LD_CG = 2 };
+// one pair of a tube of the batch (planes of stride ps)
+struct Geo {
+    int idx0;            // first cell
+    int x0;
+    bool has1;           // x0 + 1 is inside the tube
+    int oa, oc;          // offsets of the pairs holding x0-2, x0-1 and x0+2, x0+3
+    unsigned xfix;       // XF_*
+};
+
+// Load kinds of the batch.  LD_CA (cached in L1) when only threads of the
+// same block wrote the data (ordered by the block barrier), LD_CG (cached in
+// L2 only) when other blocks of the cluster wrote it on other SMs.
+enum { LD_CA = 1, LD_CG = 2 };
 template <int LD>
 __device__ __forceinline__ f2 ld2(const float *q)
 {
     const float2 *p = reinterpret_cast<const float2 *>(q);
     float2 v;
     if constexpr (LD == LD_CG) v = __ldcg(p);
-    else if constexpr (LD == LD_CA) v = __ldca(p);
-    else v = __ldg(p);
+    else v = __ldca(p);
     return f2{v.x, v.y};
 }
-template <int LD>
-__device__ __forceinline__ float ld1(const float *q)
-{
-    if constexpr (LD == LD_CG) return __ldcg(q);
-    else if constexpr (LD == LD_CA) return __ldca(q);
-    else return __ldg(q);
-}
 
-// the pair of cells (x0, x0+1) at element offset `off` from idx0
-template <bool VEC2, int LD = LD_NC>
-__device__ __forceinline__ f2 ldpair(const float *q, const Geo &g, int off)
-{
-    if constexpr (VEC2) return ld2<LD>(q + g.idx0 + off);
-    else return f2{ld1<LD>(q + g.idx0 + off), ld1<LD>(q + g.idx1 + off)};
-}
-
-template <bool VEC2>
-__device__ __forceinline__ void stpair(float *q, const Geo &g, f2 v)
-{
-    if constexpr (VEC2) {
-        *reinterpret_cast<float2 *>(q + g.idx0) = make_float2(v.x, v.y);
-    } else {
-        q[g.idx0] = v.x;
-        if (g.has1) q[g.idx1] = v.y;
-    }
-}
-
-// one value of the x-stencil through the boundary map (odd nx only)
-static __device__ __noinline__ float xval_mapped(const float *q, int idx0, int x0, int k, const StepParams &p,
-                                          float ghost)
-{
-    bool gh;
-    const int c = map1(x0 - 2 + k, p.nx, p.bc_lo[0], p.bc_hi[0], gh);
-    return gh ? ghost : __ldg(q + idx0 + (c - x0));
-}
-
-// Where the stencil values of one population come from: straight from global
-// memory (GlobalSrc), or from this thread's shared-memory staging slots that
-// asynchronous copies filled earlier (StageSrc).  get(slot, off) returns the
-// pair at element offset `off` from idx0; `slot` is its staging slot: 0, 1, 2
-// for x0-2, x0, x0+2, then 3 + 3 (A - 1) + k for the k-th neighbour pair along
-// axis A (see stage_item).
-template <bool VEC2, int LD>
-struct GlobalSrc {
-    const float *q;
-    const Geo &g;
-    __device__ __forceinline__ f2 get(int, int off) const { return ldpair<VEC2, LD>(q, g, off); }
-    template <int A, int D>
-    __device__ __forceinline__ f2 nb(int slot, int off) const { return get(slot, off); }
-};
-
+// Where the stencil values of one population come from.  get(slot): the pairs
+// at x0-2, x0, x0+2 (slots 0, 1, 2); nb<A, D>(slot): the pair at distance D
+// along axis A, the k-th one that population needs there (slot 3 A + k).
 struct StageSrc {
-    const f2 *s;     // slot 0 of this thread's buffer
+    const f2 *s;     // slot 0 of this thread's shared-memory buffer
     int stride;      // f2 elements between slots
-    __device__ __forceinline__ f2 get(int slot, int) const { return s[slot * stride]; }
+    __device__ __forceinline__ f2 get(int slot) const { return s[slot * stride]; }
     template <int A, int D>
-    __device__ __forceinline__ f2 nb(int slot, int off) const { return get(slot, off); }
+    __device__ __forceinline__ f2 nb(int slot) const { return get(slot); }
+    __device__ __forceinline__ float extra() const { return 0.0f; }
 };
-// TileSrc (rlb_bulk.cuh): the block's bulk-copied tiles; it takes the
-// neighbours along y and z by axis and distance, the x pairs by slot
+// values loaded into registers
+struct Sten {
+    f2 v[9];
+    float ex;
+};
+struct RegSrc {
+    const Sten &s;
+    __device__ __forceinline__ f2 get(int slot) const { return s.v[slot]; }
+    template <int A, int D>
+    __device__ __forceinline__ f2 nb(int slot) const { return s.v[slot]; }
+    __device__ __forceinline__ float extra() const { return s.ex; }
+};
+// TileSrc (rlb_bulk.cuh): the block's bulk-copied tiles
 
-// x0-2 .. x0+3 of one plane.  With even nx every thread loads three aligned
-// pairs; periodic edges wrap to aligned pairs, and the clamped (open) or ghost
-// (inlet) positions of the two edge columns are patched afterwards.
-template <bool VEC2, int LD, typename Src>
-__device__ __forceinline__ void xstencil(const Src &src, const float *q, const Geo &g, const StepParams &p,
-                                         float ghost, float (&v)[6])
+// x0-2 .. x0+3 of one population: three aligned pairs, patched at a row's ends
+template <bool ODDP, typename Src>
+__device__ __forceinline__ void xstencil(const Src &src, unsigned xfix, float ghost, float (&v)[6])
 {
-    if constexpr (VEC2) {
-        const f2 a = src.get(0, g.oa), b = src.get(1, 0), c = src.get(2, g.oc);
-        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y; v[4] = c.x; v[5] = c.y;
-        if (g.xfix) {
-            if (g.xfix & XF_LO_CLAMP) { v[0] = v[2]; v[1] = v[2]; }
-            if (g.xfix & XF_LO_GHOST) { v[0] = ghost; v[1] = ghost; }
-            if (g.xfix & XF_HI_CLAMP) { v[4] = v[3]; v[5] = v[3]; }
-            if (g.xfix & XF_HI_GHOST) { v[4] = ghost; v[5] = ghost; }
-            if (g.xfix & XF_HI_ODD1) { v[3] = v[2]; v[4] = v[2]; v[5] = v[2]; }
-            if (g.xfix & XF_HI_ODD3) v[5] = v[4];
+    const f2 a = src.get(0), b = src.get(1), c = src.get(2);
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y; v[4] = c.x; v[5] = c.y;
+    if (xfix) {
+        if (xfix & XF_LO_CLAMP) { v[0] = v[2]; v[1] = v[2]; }
+        if (xfix & XF_LO_GHOST) { v[0] = ghost; v[1] = ghost; }
+        if (xfix & XF_HI_CLAMP) { v[4] = v[3]; v[5] = v[3]; }
+        if (xfix & XF_HI_GHOST) { v[4] = ghost; v[5] = ghost; }
+        if (xfix & XF_HI_ODD1) { v[3] = v[2]; v[4] = v[2]; v[5] = v[2]; }
+        if (xfix & XF_HI_ODD3) v[5] = v[4];
+        if (xfix & XF_HI_ODD1G) { v[3] = ghost; v[4] = ghost; v[5] = ghost; }
+        if (xfix & XF_HI_ODD3G) v[5] = ghost;
+        if constexpr (ODDP) {
+            if (xfix & XF_LO_EX) { v[0] = v[1]; v[1] = src.extra(); }
+            if (xfix & XF_HI_EX) v[5] = src.extra();
+            if (xfix & XF_HI_WRAP1) { v[3] = v[4]; v[4] = v[5]; }
+            if (xfix & XF_HI_SELF) v[5] = v[2];
         }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) v[k] = xval_mapped(q, g.idx0, g.x0, k, p, ghost);
     }
-}
-
-// element offset of the row (A = 1) or plane (A = 2) at distance d
-template <int A>
-__device__ __forceinline__ int off_of(const Geo &g, const StepParams &p, int d)
-{
-    const int k = d < 0 ? d + 2 : d + 1;
-    if constexpr (A == 1) return g.yoff[k];
-    else return g.zoff[k];
 }
 
 // Divisions and the logarithm of the per-cell scalar work (recovery, tau,
@@ -338,6 +306,50 @@ __device__ __forceinline__ f2 eq2(const W2 &e)
     }
 }
 
+// The coefficients as the update takes them from this thread's shared-memory
+// slots (slot k at q[k * stride]): the rest value, then per axis the even part
+// a0 + ad and the odd part ab, then per plane (xy, xz, yz) the even part
+// d0 + (dd_a + dd_b), the odd parts db per axis and dk per plane.  They are
+// read where a population needs them and hold no registers between.
+constexpr int kEqSlots = 16;
+__device__ __forceinline__ void park_eq(const W2 &e, f2 *q, int stride)
+{
+    q[0] = e.r0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        q[(1 + j) * stride] = e.a0 + e.ad[j];
+        q[(4 + j) * stride] = e.ab[j];
+        q[(10 + j) * stride] = e.db[j];
+        q[(13 + j) * stride] = e.dk[j];
+    }
+    q[7 * stride] = e.d0 + (e.dd[0] + e.dd[1]);
+    q[8 * stride] = e.d0 + (e.dd[0] + e.dd[2]);
+    q[9 * stride] = e.d0 + (e.dd[1] + e.dd[2]);
+}
+template <int I>
+__device__ __forceinline__ f2 eq_parked(const f2 *q, int stride)
+{
+    constexpr int cx = cdir<I, 0>(), cy = cdir<I, 1>(), cz = cdir<I, 2>();
+    constexpr int sh = shell<I>();
+    if constexpr (sh == 0) {
+        return q[0];
+    } else if constexpr (sh == 1) {
+        constexpr int a = cx != 0 ? 0 : (cy != 0 ? 1 : 2);
+        const f2 base = q[(1 + a) * stride], b = q[(4 + a) * stride];
+        return cx + cy + cz > 0 ? base + b : base - b;
+    } else {
+        constexpr int a = cx != 0 ? 0 : 1;
+        constexpr int b = cz != 0 ? 2 : 1;
+        constexpr int ca = a == 0 ? cx : cy, cb = b == 2 ? cz : cy;
+        constexpr int ko = (a == 0 && b == 1) ? 0 : ((a == 0 && b == 2) ? 1 : 2);
+        f2 v = q[(7 + ko) * stride];
+        const f2 da = q[(10 + a) * stride], db = q[(10 + b) * stride], dk = q[(13 + ko) * stride];
+        v = ca > 0 ? v + da : v - da;
+        v = cb > 0 ? v + db : v - db;
+        return ca * cb > 0 ? v + dk : v - dk;
+    }
+}
+
 // Landau-frame recovery of a pair from the raw sums S = sum f, V_a = sum c_a f
 // (double-float) and Sh = sum h: E = xi0^2 S, M = xi0 V,
 // E^2 - |M|^2 = xi0^2 (xi0^2 S^2 - |V|^2) formed in double-float,
@@ -413,8 +425,8 @@ __device__ __forceinline__ float tau1(float P, float n, float eta_over_s)
 
 // streaming increment of population I along axis A for the pair (+ bulk lap)
 template <bool IS_F, int I, int A, int LAT, typename Src>
-__device__ __forceinline__ void axis2(const Src &src, const Geo &g, const StepParams &p, const float (&xv)[6],
-                                      f2 C, float k1, float k2, float hl, f2 &inc, f2 &lap)
+__device__ __forceinline__ void axis2(const Src &src, const float (&xv)[6], f2 C, float k1, float k2, float hl,
+                                      f2 &inc, f2 &lap)
 {
     constexpr int sb = 3 * A;   // first staging slot of axis A (A = 1, 2)
     constexpr int c = cdir<I, A, LAT>();
@@ -439,50 +451,218 @@ __device__ __forceinline__ void axis2(const Src &src, const Geo &g, const StepPa
         }
     } else {
         if constexpr (c > 0) {
-            const f2 Aq = src.template nb<A, -2>(sb, off_of<A>(g, p, -2));
-            const f2 B = src.template nb<A, -1>(sb + 1, off_of<A>(g, p, -1));
-            const f2 Dq = src.template nb<A, 1>(sb + 2, off_of<A>(g, p, 1));
+            const f2 Aq = src.template nb<A, -2>(sb);
+            const f2 B = src.template nb<A, -1>(sb + 1);
+            const f2 Dq = src.template nb<A, 1>(sb + 2);
             const f2 d0 = B - Aq, d1 = C - B, d2 = Dq - C;
             const f2 Dv = fma2(bc(hl), mm(d2, d1) - mm(d1, d0), d1);
             inc = fma2(bc(-k), Dv, inc);
             if constexpr (need_lap) lap = lap + (d2 - d1);
         } else if constexpr (c < 0) {
-            const f2 B = src.template nb<A, -1>(sb, off_of<A>(g, p, -1));
-            const f2 Dq = src.template nb<A, 1>(sb + 1, off_of<A>(g, p, 1));
-            const f2 Eq = src.template nb<A, 2>(sb + 2, off_of<A>(g, p, 2));
+            const f2 B = src.template nb<A, -1>(sb);
+            const f2 Dq = src.template nb<A, 1>(sb + 1);
+            const f2 Eq = src.template nb<A, 2>(sb + 2);
             const f2 e0 = C - B, e1 = Dq - C, e2 = Eq - Dq;
             const f2 Dv = fma2(bc(-hl), mm(e1, e2) - mm(e0, e1), e1);
             inc = fma2(bc(k), Dv, inc);
             if constexpr (need_lap) lap = lap + (e1 - e0);
         } else if constexpr (need_lap) {
-            const f2 B = src.template nb<A, -1>(sb, off_of<A>(g, p, -1));
-            const f2 Dq = src.template nb<A, 1>(sb + 1, off_of<A>(g, p, 1));
+            const f2 B = src.template nb<A, -1>(sb);
+            const f2 Dq = src.template nb<A, 1>(sb + 1);
             lap = lap + ((Dq - C) - (C - B));
         }
     }
 }
 
 // f (or h) + streaming (+ bulk) of population I for the pair: the explicit part of Eq. 57
-template <int DIM, bool IS_F, int I, bool VEC2, int LD, int LAT, typename Src>
-__device__ __forceinline__ f2 streamed2(const Src &src, const float *q, const Geo &g, const StepParams &p,
-                                        float ghost, float k1, float k2, float hl, float kb)
+template <int DIM, bool IS_F, int I, int LAT, bool ODDP, typename Src>
+__device__ __forceinline__ f2 streamed2(const Src &src, unsigned xfix, float ghost, float k1, float k2, float hl,
+                                        float kb)
 {
     constexpr bool xneed = cdir<I, 0, LAT>() != 0 || (IS_F && I != 0);
     float xv[6];
     f2 C;
     if constexpr (xneed) {
-        xstencil<VEC2, LD>(src, q, g, p, ghost, xv);
+        xstencil<ODDP>(src, xfix, ghost, xv);
         C = mk(xv[2], xv[3]);
     } else {
-        C = src.get(1, 0);
+        C = src.get(1);
     }
     f2 inc = bc(0.0f), lap = bc(0.0f);
-    if constexpr (xneed) axis2<IS_F, I, 0, LAT>(src, g, p, xv, C, k1, k2, hl, inc, lap);
-    if constexpr (DIM > 1) axis2<IS_F, I, 1, LAT>(src, g, p, xv, C, k1, k2, hl, inc, lap);
-    if constexpr (DIM > 2) axis2<IS_F, I, 2, LAT>(src, g, p, xv, C, k1, k2, hl, inc, lap);
+    if constexpr (xneed) axis2<IS_F, I, 0, LAT>(src, xv, C, k1, k2, hl, inc, lap);
+    if constexpr (DIM > 1) axis2<IS_F, I, 1, LAT>(src, xv, C, k1, k2, hl, inc, lap);
+    if constexpr (DIM > 2) axis2<IS_F, I, 2, LAT>(src, xv, C, k1, k2, hl, inc, lap);
     if constexpr (IS_F && I != 0) inc = fma2(bc(kb), lap, inc);
     return C + inc;
 }
+
+// ---------------------------------------------------------------------------
+// Sources and destinations of one pair's update (the IO of update_pair).  An
+// item is one class of f (J < NP) or of h (J - NP):
+//   begin()          start the loads of the first items' stencils
+//   own<J>()         the pair's own populations
+//   pre<S, J>()      the explicit part (streamed2) of item J, the S-th taken
+//   put<J>(v)        the new populations
+//   prev<K>(), put_prev<K>(v)   the previous level's K-th value
+// ---------------------------------------------------------------------------
+template <int NP, int J>
+struct Item {
+    static constexpr bool IS_F = J < NP;
+    static constexpr int I = rep<NP>(IS_F ? J : J - NP);
+    static constexpr int K = IS_F ? I : 19 + I;   // population of the block
+};
+
+// The order in which update_pair takes the items: f then h; in Euler mode f
+// and h of each class in turn
+template <bool EULER, int NP>
+constexpr int item_at(int s)
+{
+    return EULER ? (s % 2 ? NP + s / 2 : s / 2) : s;
+}
+
+// Grids: stencils straight from global memory into registers, kAhead items
+// before their use.  Staging them through shared memory by cp.async (two items
+// ahead) took 74 % of the L1 data path's wavefronts: every value went through
+// it three times.  Distance measured on the 512 x 256 x 256 and 2048 x 1024
+// shock-clouds, ms a step at 1 / 2 / 3 / 4 items: 4.29 / 3.78 / 3.55 / 3.97
+// and 0.199 / 0.190 / 0.177 / 0.183 (4 items spill); an L2 prefetch of the
+// rows ahead on top measured slower (3.59 to 3.76 ms, 0.180 to 0.205 ms).
+template <int DIM, bool EULER, int NP, int LAT, bool ODDP>
+struct BlockIO {
+    const StepParams &p;
+    const char *c, *l, *r;        // population 0 of the pairs at x0, x0-2, x0+2 (mapped)
+    const char *y[4], *z[4];      // of the rows at y-2, y-1, y+1, y+2 and the planes at z-2 .. z+2 (mapped)
+    const char *e;                // ODDP: of the extra value (XF_LO_EX, XF_HI_EX)
+    char *o;                      // of the pair in the buffer written
+    float *pv;                    // previous level of the pair
+    unsigned xfix;
+    float kb;
+    static constexpr int kAhead = EULER ? 2 : (DIM == 1 ? 4 : 3);
+    Sten st[kAhead + 1];
+
+    static constexpr int NI = 2 * NP;
+
+    template <int K>
+    static __device__ __forceinline__ f2 ld(const char *q)
+    {
+        f2 v;
+        asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2+%3];" : "=f"(v.x), "=f"(v.y) : "l"(q), "n"(K * kBlk * 4));
+        return v;
+    }
+    template <int J>
+    __device__ __forceinline__ void load(Sten &s) const
+    {
+        using T = Item<NP, J>;
+        constexpr bool need_lap = T::IS_F && T::I != 0;
+        constexpr int cx = cdir<T::I, 0, LAT>(), cy = cdir<T::I, 1, LAT>(), cz = cdir<T::I, 2, LAT>();
+        if constexpr (cx != 0 || need_lap) {
+            s.v[0] = ld<T::K>(l);
+            s.v[2] = ld<T::K>(r);
+            if constexpr (ODDP) {
+                s.ex = 0.0f;
+                if (xfix & (XF_LO_EX | XF_HI_EX)) s.ex = __ldg(reinterpret_cast<const float *>(e) + T::K * kBlk);
+            }
+        }
+        s.v[1] = ld<T::K>(c);
+        auto axis = [&](auto ac, const char *const (&q)[4]) {
+            constexpr int A = decltype(ac)::value;
+            constexpr int cc = A == 1 ? cy : cz;
+            if constexpr (cc > 0) {
+                s.v[3 * A] = ld<T::K>(q[0]);
+                s.v[3 * A + 1] = ld<T::K>(q[1]);
+                s.v[3 * A + 2] = ld<T::K>(q[2]);
+            } else if constexpr (cc < 0) {
+                s.v[3 * A] = ld<T::K>(q[1]);
+                s.v[3 * A + 1] = ld<T::K>(q[2]);
+                s.v[3 * A + 2] = ld<T::K>(q[3]);
+            } else if constexpr (need_lap) {
+                s.v[3 * A] = ld<T::K>(q[1]);
+                s.v[3 * A + 1] = ld<T::K>(q[2]);
+            }
+        };
+        if constexpr (DIM > 1) axis(std::integral_constant<int, 1>{}, y);
+        if constexpr (DIM > 2) axis(std::integral_constant<int, 2>{}, z);
+    }
+    __device__ __forceinline__ void begin()
+    {
+        for_pops(std::make_integer_sequence<int, kAhead>{}, [&](auto sc) {
+            constexpr int S = decltype(sc)::value;
+            load<item_at<EULER, NP>(S)>(st[S]);
+        });
+    }
+    template <int J>
+    __device__ __forceinline__ f2 own() const
+    {
+        const float2 v = __ldg(reinterpret_cast<const float2 *>(c + Item<NP, J>::K * kBlk * 4));
+        return f2{v.x, v.y};
+    }
+    template <int S, int J>
+    __device__ __forceinline__ f2 pre()
+    {
+        using T = Item<NP, J>;
+        if constexpr (S + kAhead < NI) load<item_at<EULER, NP>(S + kAhead)>(st[(S + kAhead) % (kAhead + 1)]);
+        const RegSrc src{st[S % (kAhead + 1)]};
+        return streamed2<DIM, T::IS_F, T::I, LAT, ODDP>(src, xfix, T::IS_F ? p.f_ghost_f[T::I] : p.f_ghost_h[T::I],
+                                                        p.f_k1, p.f_k2, p.f_half_lim, kb);
+    }
+    template <int J>
+    __device__ __forceinline__ void put(f2 v) const
+    {
+        *reinterpret_cast<float2 *>(o + Item<NP, J>::K * kBlk * 4) = make_float2(v.x, v.y);
+    }
+    template <int K>
+    __device__ __forceinline__ f2 prev() const
+    {
+        const float2 v = *reinterpret_cast<const float2 *>(pv + K * kBlk);
+        return f2{v.x, v.y};
+    }
+    template <int K>
+    __device__ __forceinline__ void put_prev(f2 v) const
+    {
+        *reinterpret_cast<float2 *>(pv + K * kBlk) = make_float2(v.x, v.y);
+    }
+};
+
+// Planes of stride ps (the batch's tubes and the bulk-staged grids): the own
+// pair and the previous level
+template <int NP, int LD>
+struct PlaneIO {
+    const StepParams &p;
+    const float *f, *h;
+    float *fo, *ho, *pv;
+    long long ps;
+    int idx0;
+    unsigned xfix;
+    float kb;
+    template <int J>
+    __device__ __forceinline__ f2 own() const
+    {
+        const float *q = (Item<NP, J>::IS_F ? f : h) + Item<NP, J>::I * ps + idx0;
+        if constexpr (LD == 0) {
+            const float2 v = __ldg(reinterpret_cast<const float2 *>(q));
+            return f2{v.x, v.y};
+        } else {
+            return ld2<LD>(q);
+        }
+    }
+    template <int J>
+    __device__ __forceinline__ void put(f2 v) const
+    {
+        float *q = (Item<NP, J>::IS_F ? fo : ho) + Item<NP, J>::I * ps + idx0;
+        *reinterpret_cast<float2 *>(q) = make_float2(v.x, v.y);
+    }
+    template <int K>
+    __device__ __forceinline__ f2 prev() const
+    {
+        const float2 v = *reinterpret_cast<const float2 *>(pv + K * ps + idx0);
+        return f2{v.x, v.y};
+    }
+    template <int K>
+    __device__ __forceinline__ void put_prev(f2 v) const
+    {
+        *reinterpret_cast<float2 *>(pv + K * ps + idx0) = make_float2(v.x, v.y);
+    }
+};
 
 // Asynchronous copies (cp.async, cached in L1) into shared memory, completed
 // per thread by cp.async.wait_group: no other thread reads the slots.
@@ -496,185 +676,122 @@ __device__ __forceinline__ void cp_wait()
 {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-
-#ifndef RLB_STAGE_BUFS
-#define RLB_STAGE_BUFS 3
-#endif
-// pairs staged per population: 3 along x, 3 along each other streamed axis
-template <int DIM>
-constexpr int stage_slots()
-{
-    return 3 * DIM;
-}
-constexpr int kStageBufs = RLB_STAGE_BUFS;   // populations in flight: the one computed and the next ones
+constexpr int kStageBufs = 3;                // populations in flight: the one computed and the next ones
 constexpr int kStageAhead = kStageBufs - 1;  // prefetch distance in populations
 
-// Issue the copies of item J (J < NP: f class J, else h class J - NP) into
-// staging buffer J % kStageBufs: the same pairs, in the same
-// slots, that streamed2 reads through StageSrc.  dst0 = shared address of
-// slot 0 of buffer 0 of this thread, sstride = bytes between slots.
-template <int DIM, int NP, int J, int LAT>
-__device__ __forceinline__ void stage_item(const float *f, const float *h, const Geo &g, const StepParams &p,
-                                           long long ps, unsigned dst0, unsigned sstride)
-{
-    constexpr bool IS_F = J < NP;
-    constexpr int I = rep<NP>(IS_F ? J : J - NP);
-    constexpr bool xneed = cdir<I, 0, LAT>() != 0 || (IS_F && I != 0);
-    constexpr bool need_lap = IS_F && I != 0;
-    const unsigned d = dst0 + unsigned(J % kStageBufs) * stage_slots<DIM>() * sstride;
-    if constexpr (DIM == 3) {
-        // one population plane base for the block, the thread's fixed byte
-        // offsets on top (fewer address instructions than a per-thread base)
-        const char *qb = reinterpret_cast<const char *>((IS_F ? f : h) + I * ps);
-        auto at = [&](int s) { return reinterpret_cast<const float *>(qb + g.sb[s]); };
+// Tubes of the batch: the three pairs of each population's stencil are copied
+// into this thread's shared-memory slots kStageAhead populations ahead of
+// their use.  stage = slot 0 of buffer 0 of this thread, sstride = f2
+// elements between slots.
+template <int NP, int LD>
+struct StageIO : PlaneIO<NP, LD> {
+    int oa, oc;
+    f2 *stage;
+    int sstride;
+    unsigned dst0;
+
+    static constexpr int NI = 2 * NP;
+    template <int J>
+    __device__ __forceinline__ void issue() const
+    {
+        using T = Item<NP, J>;
+        constexpr bool xneed = cdir<T::I, 0>() != 0 || (T::IS_F && T::I != 0);
+        const unsigned ss = unsigned(sstride * sizeof(f2));
+        const unsigned d = dst0 + unsigned(J % kStageBufs) * 3 * ss;
+        const float *q = (T::IS_F ? this->f : this->h) + T::I * this->ps + this->idx0;
         if constexpr (xneed) {
-            cp8(d + 0 * sstride, at(0));
-            cp8(d + 2 * sstride, at(2));
+            cp8(d, q + oa);
+            cp8(d + 2 * ss, q + oc);
         }
-        cp8(d + 1 * sstride, at(1));
-        auto axis = [&](auto ac) {
-            constexpr int A = decltype(ac)::value;
-            constexpr int c = cdir<I, A, LAT>();
-            constexpr int s0 = 3 + 4 * (A - 1);   // slots of distances -2, -1, +1, +2
-            const unsigned b = d + unsigned(3 * A) * sstride;
-            if constexpr (c > 0) {
-                cp8(b, at(s0 + 0));
-                cp8(b + sstride, at(s0 + 1));
-                cp8(b + 2 * sstride, at(s0 + 2));
-            } else if constexpr (c < 0) {
-                cp8(b, at(s0 + 1));
-                cp8(b + sstride, at(s0 + 2));
-                cp8(b + 2 * sstride, at(s0 + 3));
-            } else if constexpr (need_lap) {
-                cp8(b, at(s0 + 1));
-                cp8(b + sstride, at(s0 + 2));
-            }
-        };
-        axis(std::integral_constant<int, 1>{});
-        axis(std::integral_constant<int, 2>{});
+        cp8(d + ss, q);
         cp_commit();
-        return;
     }
-    const float *q = (IS_F ? f : h) + I * ps + g.idx0;
-    if constexpr (xneed) {
-        cp8(d + 0 * sstride, q + g.oa);
-        cp8(d + 2 * sstride, q + g.oc);
+    __device__ __forceinline__ void begin()
+    {
+        dst0 = unsigned(__cvta_generic_to_shared(stage));
+        for_pops(std::make_integer_sequence<int, kStageAhead>{}, [&](auto jc) { issue<decltype(jc)::value>(); });
     }
-    cp8(d + 1 * sstride, q);
-    auto axis = [&](auto ac) {
-        constexpr int A = decltype(ac)::value;
-        constexpr int c = cdir<I, A, LAT>();
-        const unsigned b = d + unsigned(3 * A) * sstride;
-        if constexpr (c > 0) {
-            cp8(b, q + off_of<A>(g, p, -2));
-            cp8(b + sstride, q + off_of<A>(g, p, -1));
-            cp8(b + 2 * sstride, q + off_of<A>(g, p, 1));
-        } else if constexpr (c < 0) {
-            cp8(b, q + off_of<A>(g, p, -1));
-            cp8(b + sstride, q + off_of<A>(g, p, 1));
-            cp8(b + 2 * sstride, q + off_of<A>(g, p, 2));
-        } else if constexpr (need_lap) {
-            cp8(b, q + off_of<A>(g, p, -1));
-            cp8(b + sstride, q + off_of<A>(g, p, 1));
+    template <int S, int J>
+    __device__ __forceinline__ f2 pre()
+    {
+        using T = Item<NP, J>;
+        if constexpr (J + kStageAhead < NI) {
+            issue<J + kStageAhead>();
+            cp_wait<kStageAhead>();
+        } else {
+            cp_wait<NI - 1 - J>();   // the groups issued after item J's
         }
-    };
-    if constexpr (DIM > 1) axis(std::integral_constant<int, 1>{});
-    if constexpr (DIM > 2) axis(std::integral_constant<int, 2>{});
-    cp_commit();
-}
+        const StageSrc src{stage + (J % kStageBufs) * 3 * sstride, sstride};
+        return streamed2<1, T::IS_F, T::I, 0, false>(src, this->xfix, 0.0f, this->p.f_k1, this->p.f_k2,
+                                                     this->p.f_half_lim, this->kb);
+    }
+};
+
+// 3-D grids staged by bulk copies (rlb_bulk.cuh)
+template <int LAT>
+struct BulkIO : PlaneIO<19, 0> {
+    Bulk *bk;
+    static constexpr int NP = 19, NI = 38;
+    __device__ __forceinline__ void begin() {}
+    template <int S, int J>
+    __device__ __forceinline__ f2 pre()
+    {
+        using T = Item<NP, J>;
+        constexpr int b = J % kBulkBufs;
+        constexpr unsigned par = unsigned(J / kBulkBufs) & 1u;
+        if (!bk->failed && !mbar_wait(&bk->full[b], par)) {
+            bk->failed = true;
+            atomicOr(p.status, unsigned(ST_TIMEOUT));
+        }
+        bk->failed = __any_sync(0xffffffffu, bk->failed);   // warp-uniform: the issue below is warp-wide
+        const TileSrc src{bk->ctr + b * kTileFloats, bk->zpl + b * kTileFloats};
+        const f2 r = streamed2<3, T::IS_F, T::I, LAT, false>(src, xfix, T::IS_F ? p.f_ghost_f[T::I] : p.f_ghost_h[T::I],
+                                                             p.f_k1, p.f_k2, p.f_half_lim, kb);
+        // this warp is done with buffer b: it counts itself out, and the
+        // warp that counts the last of the 8 refills the buffer with item
+        // J + kBulkBufs (release fence before the count, acquire after
+        // it, then the generic-to-async proxy fence before the copies
+        // overwrite what the other warps read)
+        if constexpr (J + kBulkBufs < NI) {
+            __syncwarp();
+            int last = 0;
+            if (bk->lane == 0) {
+                asm volatile("fence.acq_rel.cta;" ::: "memory");
+                last = (atomicAdd(&bk->done[b], 1) & 7) == 7;
+                if (last) asm volatile("fence.acq_rel.cta;" ::: "memory");
+            }
+            if (__shfl_sync(0xffffffffu, last, 0) && !bk->failed) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                bulk_issue<NP, J + kBulkBufs, LAT>(*bk, p, f, h);
+            }
+        }
+        return r;
+    }
+};
 
 // The update of one pair of cells (Eq. 57 for f and h), shared by the grid
-// kernel and the batched tube kernel.  eos = eta/s and kb = the bulk
-// prefactor of the cell's grid or tube.
+// kernels and the batched tube kernel.  io: where its values come from and go
+// to (above); has1: the pair's second cell is inside the grid; eos = eta/s of
+// the cell's grid or tube.
 //
-// park (PARK = true): this thread's slots in shared memory, slot k at
-// park[k * pstride]; the h-equilibrium coefficients wait there while the f
-// populations are updated, which frees their registers for the f loop.
-//
-// stage (STAGE = true, even nx, viscous step): the stencil of each population
-// is copied asynchronously into this thread's shared-memory slots
-// kStageAhead populations ahead of its use (stage_item), so that the loads of the next
-// populations are in flight while one is computed; stage = slot 0 of buffer
-// 0 of this thread, sstride = f2 elements between slots.
+// park (viscous step): this thread's slots in shared memory, slot k at
+// park[k * pstride]: the h-equilibrium coefficients wait there while the f
+// populations are updated (kParkH slots), and with PARKF the coefficients in
+// use too (kEqSlots more), which leaves their registers to the stencils in
+// flight.  Grids of 2 and 3 dimensions take PARKF (3-D: 3.58 ms a step with
+// three items in flight; with the f coefficients in registers one item fits,
+// 4.15 ms); in one dimension an item is three pairs and registers suffice.
 //
 // NP = 7 or 14: the 1-D or 2-D symmetry reduction (see rep and mult); only
-// the planes of the class representatives are read and written, and the
-// previous level's planes of the zero sums (sum c_z f; 1-D also sum c_y f)
-// are left alone.
-template <int DIM, bool EULER, bool VEC2, int LD = LD_NC, bool PARK = false, bool STAGE = false, int NP = 19,
-          int LAT = 0, bool REC64 = false, bool BULK = false>
-__device__ __forceinline__ void update_pair(const StepParams &p, const Geo &g, float eos, float kb,
-                                            const float *__restrict__ f, const float *__restrict__ h,
-                                            float *__restrict__ fo, float *__restrict__ ho,
-                                            float *__restrict__ prev, long long ps,
-                                            f2 *park = nullptr, int pstride = 0,
-                                            f2 *stage = nullptr, int sstride = 0, Bulk *bk = nullptr)
+// the class representatives are read and written, and the previous level's
+// zero sums (sum c_z f; 1-D also sum c_y f) are left alone.
+template <bool EULER, bool PARKF, int NP, int LAT, bool REC64, typename IO>
+__device__ __forceinline__ void update_pair(const StepParams &p, IO &io, bool has1, float eos, f2 *park = nullptr,
+                                            int pstride = 0)
 {
-    const float k1 = p.f_k1, k2 = p.f_k2, hl = p.f_half_lim;
-    static_assert(!STAGE || (VEC2 && !EULER), "staging needs aligned pairs and the viscous step");
-    static_assert(NP == 19 || (NP == 7 && DIM == 1 && !EULER) || (NP == 14 && DIM == 2 && !EULER),
-                  "the symmetry reductions are 1-D or 2-D and viscous");
+    static_assert(NP == 19 || !EULER, "the symmetry reductions are viscous");
     static_assert(!REC64 || (!EULER && NP == 19), "the FP64 recovery is a variant of the viscous 19-population step");
-    static_assert(!BULK || (DIM == 3 && VEC2 && !EULER && NP == 19 && !STAGE),
-                  "bulk-copied tiles: the viscous 3-D step with aligned pairs");
-    constexpr int NI = 2 * NP;   // items: f classes, then h classes
-    unsigned sdst0 = 0;
-    if constexpr (STAGE) {
-        sdst0 = unsigned(__cvta_generic_to_shared(stage));
-        for_pops(std::make_integer_sequence<int, kStageAhead>{}, [&](auto jc) {
-            stage_item<DIM, NP, decltype(jc)::value, LAT>(f, h, g, p, ps, sdst0, unsigned(sstride * sizeof(f2)));
-        });
-    }
-    // the explicit part of item J (J < NP: f class J, else h class J - NP)
-    auto item = [&](auto jc) -> f2 {
-        constexpr int J = decltype(jc)::value;
-        constexpr bool IS_F = J < NP;
-        constexpr int I = rep<NP>(IS_F ? J : J - NP);
-        const float *q = (IS_F ? f : h) + I * ps;
-        const float ghost = IS_F ? p.f_ghost_f[I] : p.f_ghost_h[I];
-        if constexpr (BULK) {
-            constexpr int b = J % kBulkBufs;
-            constexpr unsigned par = unsigned(J / kBulkBufs) & 1u;
-            if (!bk->failed && !mbar_wait(&bk->full[b], par)) {
-                bk->failed = true;
-                atomicOr(p.status, unsigned(ST_TIMEOUT));
-            }
-            bk->failed = __any_sync(0xffffffffu, bk->failed);   // warp-uniform: the issue below is warp-wide
-            const TileSrc src{bk->ctr + b * kTileFloats, bk->zpl + b * kTileFloats};
-            const f2 r = streamed2<DIM, IS_F, I, VEC2, LD, LAT>(src, q, g, p, ghost, k1, k2, hl, kb);
-            // this warp is done with buffer b: it counts itself out, and the
-            // warp that counts the last of the 8 refills the buffer with item
-            // J + kBulkBufs (release fence before the count, acquire after
-            // it, then the generic-to-async proxy fence before the copies
-            // overwrite what the other warps read)
-            if constexpr (J + kBulkBufs < NI) {
-                __syncwarp();
-                int last = 0;
-                if (bk->lane == 0) {
-                    asm volatile("fence.acq_rel.cta;" ::: "memory");
-                    last = (atomicAdd(&bk->done[b], 1) & 7) == 7;
-                    if (last) asm volatile("fence.acq_rel.cta;" ::: "memory");
-                }
-                if (__shfl_sync(0xffffffffu, last, 0) && !bk->failed) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    bulk_issue<NP, J + kBulkBufs, LAT>(*bk, p, f, h);
-                }
-            }
-            return r;
-        } else if constexpr (STAGE) {
-            if constexpr (J + kStageAhead < NI) {
-                stage_item<DIM, NP, J + kStageAhead, LAT>(f, h, g, p, ps, sdst0, unsigned(sstride * sizeof(f2)));
-                cp_wait<kStageAhead>();
-            } else {
-                cp_wait<NI - 1 - J>();   // the groups issued after item J's
-            }
-            const StageSrc src{stage + (J % kStageBufs) * stage_slots<DIM>() * sstride, sstride};
-            return streamed2<DIM, IS_F, I, VEC2, LD, LAT>(src, q, g, p, ghost, k1, k2, hl, kb);
-        } else {
-            const GlobalSrc<VEC2, LD> src{q, g};
-            return streamed2<DIM, IS_F, I, VEC2, LD, LAT>(src, q, g, p, ghost, k1, k2, hl, kb);
-        }
-    };
+    io.begin();
 
     if constexpr (!EULER) {
         // raw sums of the local populations: S = sum f, V_a = sum c_a f
@@ -683,7 +800,7 @@ __device__ __forceinline__ void update_pair(const StepParams &p, const Geo &g, f
         for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
             constexpr int k = decltype(kc)::value;
             constexpr int I = rep<NP>(k), m = mult<NP>(k);
-            const f2 v = ldpair<VEC2, LD>(f + I * ps, g, 0);
+            const f2 v = io.template own<k>();
             // m c_i v with m and c_i powers of two: exact
             auto scaled = [&](auto wc) {
                 constexpr int w = decltype(wc)::value;
@@ -695,7 +812,7 @@ __device__ __forceinline__ void update_pair(const StepParams &p, const Geo &g, f
             // under a reduction sum c_y f (1-D) and sum c_z f are zero
             if constexpr (has_vy<NP>() && cy != 0) acc(Vy, scaled(std::integral_constant<int, cy * m>{}));
             if constexpr (has_vz<NP>() && cz != 0) acc(Vz, scaled(std::integral_constant<int, cz * m>{}));
-            const f2 hv = ldpair<VEC2, LD>(h + I * ps, g, 0);
+            const f2 hv = io.template own<NP + k>();
             acc(Hs, m == 1 ? hv : bc(float(m)) * hv);
         });
         const f2 Sh = Hs.hi + Hs.lo;
@@ -703,7 +820,7 @@ __device__ __forceinline__ void update_pair(const StepParams &p, const Geo &g, f
         Mac2 mt;
         if constexpr (REC64) mt = recover2_64<LAT>(S, Vx, Vy, Vz, Hs, ok0, ok1);
         else mt = recover2<LAT>(S, Vx, Vy, Vz, Sh, ok0, ok1);
-        if (!ok0 || (g.has1 && !ok1)) atomicOr(p.status, unsigned(ST_NONPHYSICAL));
+        if (!ok0 || (has1 && !ok1)) atomicOr(p.status, unsigned(ST_NONPHYSICAL));
 
         f2 kap;
         {
@@ -721,11 +838,11 @@ __device__ __forceinline__ void update_pair(const StepParams &p, const Geo &g, f
 
         // the previous level holds the raw moment sums of time t - dt, so the
         // targets of 2 f^eq(t) - f^eq(t - dt) are exact: T = 2 S(t) - S(t - dt)
-        const f2 Sp = ldpair<VEC2, LD>(prev + 0 * ps, g, 0);
-        const f2 Vpx = ldpair<VEC2, LD>(prev + 1 * ps, g, 0);
-        const f2 Vpy = has_vy<NP>() ? ldpair<VEC2, LD>(prev + 2 * ps, g, 0) : bc(0.0f);
-        const f2 Vpz = has_vz<NP>() ? ldpair<VEC2, LD>(prev + 3 * ps, g, 0) : bc(0.0f);
-        const f2 Shp = ldpair<VEC2, LD>(prev + 4 * ps, g, 0);
+        const f2 Sp = io.template prev<0>();
+        const f2 Vpx = io.template prev<1>();
+        const f2 Vpy = has_vy<NP>() ? io.template prev<2>() : bc(0.0f);
+        const f2 Vpz = has_vz<NP>() ? io.template prev<3>() : bc(0.0f);
+        const f2 Shp = io.template prev<4>();
         // the previous level's recovery: the same arithmetic as this level's,
         // from its stored float sums.  Its validity is not checked again: the
         // same sums passed the check as the current level one step earlier
@@ -775,45 +892,49 @@ __device__ __forceinline__ void update_pair(const StepParams &p, const Geo &g, f
             }
             const W2 ef = weigh2<Lat<LAT>::dmag>(K0, Kb, Kd, Ko, float(Lat<LAT>::w0), float(Lat<LAT>::w1), float(Lat<LAT>::w2), T0, Ta);
             // the raw sums of this level become the next step's previous level
-            stpair<VEC2>(prev + 0 * ps, g, S.hi + S.lo);
-            stpair<VEC2>(prev + 1 * ps, g, Vx.hi + Vx.lo);
-            if constexpr (has_vy<NP>()) stpair<VEC2>(prev + 2 * ps, g, Vy.hi + Vy.lo);
-            if constexpr (has_vz<NP>()) stpair<VEC2>(prev + 3 * ps, g, Vz.hi + Vz.lo);
-            stpair<VEC2>(prev + 4 * ps, g, Sh);
-            if constexpr (PARK) {
-                park[0] = H0;
-                park[10 * pstride] = T0h;
+            io.template put_prev<0>(S.hi + S.lo);
+            io.template put_prev<1>(Vx.hi + Vx.lo);
+            if constexpr (has_vy<NP>()) io.template put_prev<2>(Vy.hi + Vy.lo);
+            if constexpr (has_vz<NP>()) io.template put_prev<3>(Vz.hi + Vz.lo);
+            io.template put_prev<4>(Sh);
+            f2 *hp = park + (PARKF ? kEqSlots * pstride : 0);
+            hp[0] = H0;
+            hp[10 * pstride] = T0h;
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    park[(1 + j) * pstride] = Hb[j];
-                    park[(4 + j) * pstride] = Hd[j];
-                    park[(7 + j) * pstride] = Ho[j];
-                }
+            for (int j = 0; j < 3; ++j) {
+                hp[(1 + j) * pstride] = Hb[j];
+                hp[(4 + j) * pstride] = Hd[j];
+                hp[(7 + j) * pstride] = Ho[j];
             }
+            if constexpr (PARKF) park_eq(ef, park, pstride);
             for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
                 constexpr int k = decltype(kc)::value;
-                constexpr int I = rep<NP>(k);
-                const f2 pre = item(std::integral_constant<int, k>{});
-                stpair<VEC2>(fo + I * ps, g, fma2(kap, eq2<I>(ef) - pre, pre));
+                const f2 pre = io.template pre<k, k>();
+                f2 q;
+                if constexpr (PARKF) q = eq_parked<rep<NP>(k)>(park, pstride);
+                else q = eq2<rep<NP>(k)>(ef);
+                io.template put<k>(fma2(kap, q - pre, pre));
             });
         }
         {
-            if constexpr (PARK) {
-                H0 = park[0];
-                T0h = park[10 * pstride];
+            const f2 *hp = park + (PARKF ? kEqSlots * pstride : 0);
+            H0 = hp[0];
+            T0h = hp[10 * pstride];
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    Hb[j] = park[(1 + j) * pstride];
-                    Hd[j] = park[(4 + j) * pstride];
-                    Ho[j] = park[(7 + j) * pstride];
-                }
+            for (int j = 0; j < 3; ++j) {
+                Hb[j] = hp[(1 + j) * pstride];
+                Hd[j] = hp[(4 + j) * pstride];
+                Ho[j] = hp[(7 + j) * pstride];
             }
             const W2 eh = weigh2<Lat<LAT>::dmag>(H0, Hb, Hd, Ho, float(Lat<LAT>::wh0), float(Lat<LAT>::wh1), float(Lat<LAT>::wh2), T0h, nullptr);
+            if constexpr (PARKF) park_eq(eh, park, pstride);
             for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
                 constexpr int k = decltype(kc)::value;
-                constexpr int I = rep<NP>(k);
-                const f2 pre = item(std::integral_constant<int, NP + k>{});
-                stpair<VEC2>(ho + I * ps, g, fma2(kap, eq2<I>(eh) - pre, pre));
+                const f2 pre = io.template pre<NP + k, NP + k>();
+                f2 q;
+                if constexpr (PARKF) q = eq_parked<rep<NP>(k)>(park, pstride);
+                else q = eq2<rep<NP>(k)>(eh);
+                io.template put<NP + k>(fma2(kap, q - pre, pre));
             });
         }
     } else {
@@ -821,18 +942,18 @@ __device__ __forceinline__ void update_pair(const StepParams &p, const Geo &g, f
         df2 S{bc(0.0f), bc(0.0f)}, Vx = S, Vy = S, Vz = S, Hs = S;
         for_pops(RLB_F32_POPS, [&](auto ic) {
             constexpr int I = decltype(ic)::value;
-            const f2 v = item(std::integral_constant<int, I>{});
+            const f2 v = io.template pre<2 * I, I>();
             acc(S, v);
             constexpr int cx = cdir<I, 0, LAT>(), cy = cdir<I, 1, LAT>(), cz = cdir<I, 2, LAT>();
             if constexpr (cx != 0) acc(Vx, cx > 0 ? (cx == 1 ? v : v + v) : (cx == -1 ? -v : -(v + v)));
             if constexpr (cy != 0) acc(Vy, cy > 0 ? (cy == 1 ? v : v + v) : (cy == -1 ? -v : -(v + v)));
             if constexpr (cz != 0) acc(Vz, cz > 0 ? (cz == 1 ? v : v + v) : (cz == -1 ? -v : -(v + v)));
-            acc(Hs, item(std::integral_constant<int, 19 + I>{}));
+            acc(Hs, io.template pre<2 * I + 1, 19 + I>());
         });
         const f2 Sh = Hs.hi + Hs.lo;
         bool ok0, ok1;
         const Mac2 mt = recover2<LAT>(S, Vx, Vy, Vz, Sh, ok0, ok1);
-        if (!ok0 || (g.has1 && !ok1)) atomicOr(p.status, unsigned(ST_NONPHYSICAL));
+        if (!ok0 || (has1 && !ok1)) atomicOr(p.status, unsigned(ST_NONPHYSICAL));
         const f2 Ta[3] = {Vx.hi + Vx.lo, Vy.hi + Vy.lo, Vz.hi + Vz.lo};
         f2 K0, Kb[3], Kd[3], Ko[3];
         coef_f2<LAT>(mt, K0, Kb, Kd, Ko);
@@ -841,14 +962,14 @@ __device__ __forceinline__ void update_pair(const StepParams &p, const Geo &g, f
         const W2 eh = weigh2<Lat<LAT>::dmag>(K0, Kb, Kd, Ko, float(Lat<LAT>::wh0), float(Lat<LAT>::wh1), float(Lat<LAT>::wh2), Sh, nullptr);
         for_pops(RLB_F32_POPS, [&](auto ic) {
             constexpr int I = decltype(ic)::value;
-            stpair<VEC2>(fo + I * ps, g, eq2<I>(ef));
-            stpair<VEC2>(ho + I * ps, g, eq2<I>(eh));
+            io.template put<I>(eq2<I>(ef));
+            io.template put<19 + I>(eq2<I>(eh));
         });
-        stpair<VEC2>(prev + 0 * ps, g, S.hi + S.lo);
-        stpair<VEC2>(prev + 1 * ps, g, Ta[0]);
-        stpair<VEC2>(prev + 2 * ps, g, Ta[1]);
-        stpair<VEC2>(prev + 3 * ps, g, Ta[2]);
-        stpair<VEC2>(prev + 4 * ps, g, Sh);
+        io.template put_prev<0>(S.hi + S.lo);
+        io.template put_prev<1>(Ta[0]);
+        io.template put_prev<2>(Ta[1]);
+        io.template put_prev<3>(Ta[2]);
+        io.template put_prev<4>(Sh);
     }
 }
 
@@ -879,37 +1000,26 @@ __device__ __forceinline__ void slab_order(int slab_by, unsigned &bx, unsigned &
 #define RLB_F32_BY 8
 #endif
 
-constexpr int kParkSlots = 11;   // f2 slots per thread in shared memory
-#ifdef RLB_NO_PARK
-constexpr bool kParkOn = false;
-#else
-constexpr bool kParkOn = true;
-#endif
-#ifdef RLB_NO_STAGE
-constexpr bool kStageOn = false;
-#else
-constexpr bool kStageOn = true;
-#endif
+constexpr int kParkH = 11;   // f2 slots per thread in shared memory of the parked h coefficients
 // dynamic shared memory of one block of nthr threads
-constexpr size_t step_smem_bytes(int nthr, bool stage, int dim)
-{
-    return sizeof(f2) * size_t(nthr) * ((kParkOn ? kParkSlots : 0) + (stage ? 3 * dim * kStageBufs : 0));
-}
+constexpr size_t park_bytes(int nthr, int dim) { return sizeof(f2) * size_t(nthr) * (kParkH + (dim > 1 ? kEqSlots : 0)); }
+// the batch's blocks add the staged stencils
+constexpr size_t tube_smem_bytes(int nthr) { return sizeof(f2) * size_t(nthr) * (kParkH + 3 * kStageBufs); }
 
-// NP = 14: the 2-D symmetry reduction (DIM = 2, viscous step).  LIN: blocks
-// of one row of 32 BY threads take consecutive cell pairs t of the x-fastest
-// order (rows of ceil(nx / 2) pairs), for grids whose nx does not fill the
-// tiles; otherwise blocks of 32 x BY threads take tiles of 64 x BY cells in
-// one z-plane (the 1-D form: one row of tiles)
-template <int DIM, bool EULER, bool VEC2, int LAT, int NP = 19, bool LIN = false, bool REC64 = false>
-__global__ void __launch_bounds__(32 * RLB_F32_BY, VEC2 ? RLB_F32_MINB : 1)
-    step_f32_kernel(const StepParams p, const float *__restrict__ f, const float *__restrict__ h,
-                    float *__restrict__ fo, float *__restrict__ ho, float *__restrict__ prev)
+// NP = 14: the 2-D symmetry reduction (DIM = 2, viscous step).  ODDP: nx odd
+// with a periodic x face.  LIN: blocks of one row of 32 BY threads take
+// consecutive cell pairs t of the storage order (rows of nxe / 2 pairs), for
+// grids whose nx does not fill the tiles; otherwise blocks of 32 x BY threads
+// take tiles of 64 x BY cells in one z-plane (the 1-D form: one row of tiles)
+template <int DIM, bool EULER, bool ODDP, int LAT, int NP = 19, bool LIN = false, bool REC64 = false>
+__global__ void __launch_bounds__(32 * RLB_F32_BY, RLB_F32_MINB)
+    step_f32_kernel(const StepParams p, const float *__restrict__ f, float *__restrict__ fo, float *__restrict__ prev)
 {
     extern __shared__ f2 s_park[];
+    const int nxe = p.nx + (p.nx & 1);
     int x0, y, z;
     if constexpr (LIN) {
-        const unsigned ppr = unsigned(p.nx + 1) >> 1;
+        const unsigned ppr = unsigned(nxe) >> 1;
         const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
         const unsigned row = t / ppr;
         x0 = 2 * int(t - row * ppr);
@@ -924,43 +1034,51 @@ __global__ void __launch_bounds__(32 * RLB_F32_BY, VEC2 ? RLB_F32_MINB : 1)
         z = bz;
         if (x0 >= p.nx || y >= p.ny) return;
     }
-    const long long ps = p.ps;
+    const int i0 = x0 + nxe * (y + p.ny * z);
+    const bool has1 = x0 + 1 < p.nx;
+    const char *base = reinterpret_cast<const char *>(f);
+    auto at = [&](int i) { return base + sizeof(float) * blk_at(i); };
 
-    Geo g;
-    g.idx0 = x0 + p.nx * (y + p.ny * z);
-    g.x0 = x0;
-    g.has1 = x0 + 1 < p.nx;
-    g.idx1 = g.has1 ? g.idx0 + 1 : g.idx0;
-    g.oa = -2;
-    g.oc = 2;
-    g.xfix = 0u;
-    if (VEC2) {
-        if (x0 == 0) {   // x0-2, x0-1 are outside
-            if (p.bc_lo[0] == BC_PERIODIC) g.oa = p.nx - 2;
-            else { g.oa = 0; g.xfix |= p.bc_lo[0] == BC_OUTFLOW ? XF_LO_CLAMP : XF_LO_GHOST; }
-        }
-        if (x0 + 2 >= p.nx) {   // x0+2, x0+3 are outside
-            if (p.bc_hi[0] == BC_PERIODIC) g.oc = -x0;
-            else { g.oc = 0; g.xfix |= p.bc_hi[0] == BC_OUTFLOW ? XF_HI_CLAMP : XF_HI_GHOST; }
-        }
+    BlockIO<DIM, EULER, NP, LAT, ODDP> io{p};
+    io.c = at(i0);
+    io.o = reinterpret_cast<char *>(fo) + (io.c - base);
+    io.pv = prev + blk_prev_at(i0);
+    io.kb = p.f_kbulk;
+    // a row of one cell: the periodic neighbour is the cell itself (clamped)
+    const int lo = p.nx == 1 && p.bc_lo[0] == BC_PERIODIC ? int(BC_OUTFLOW) : p.bc_lo[0];
+    const int hi = p.nx == 1 && p.bc_hi[0] == BC_PERIODIC ? int(BC_OUTFLOW) : p.bc_hi[0];
+    int ol = -2, orr = 2;
+    unsigned xfix = 0u;
+    if (x0 == 0) {   // x0-2, x0-1 are outside
+        ol = 0;
+        if (lo != BC_PERIODIC) xfix |= lo == BC_OUTFLOW ? XF_LO_CLAMP : XF_LO_GHOST;
+        else if (ODDP) { ol = p.nx - 3; xfix |= XF_LO_EX; }
+        else ol = p.nx - 2;
     }
+    if (x0 + 2 >= p.nx) {   // x0+2, x0+3 are outside (and x0+1 at the end of an odd row)
+        orr = 0;
+        if (hi == BC_PERIODIC) {
+            orr = -x0;
+            if (ODDP && !has1) xfix |= XF_HI_WRAP1;
+        } else if (has1) {
+            xfix |= hi == BC_OUTFLOW ? XF_HI_CLAMP : XF_HI_GHOST;
+        } else {
+            xfix |= hi == BC_OUTFLOW ? XF_HI_ODD1 : XF_HI_ODD1G;
+        }
+    } else if (x0 + 3 == p.nx) {   // x0+3 is outside
+        if (hi != BC_PERIODIC) xfix |= hi == BC_OUTFLOW ? XF_HI_ODD3 : XF_HI_ODD3G;
+        else xfix |= x0 == 0 ? XF_HI_SELF : XF_HI_EX;
+    }
+    io.l = at(i0 + ol);
+    io.r = at(i0 + orr);
+    if constexpr (ODDP) io.e = at(i0 + ((xfix & XF_LO_EX) ? p.nx - 1 : ((xfix & XF_HI_EX) ? -x0 : 0)));
+    io.xfix = xfix;
     {
         const int ds[4] = {-2, -1, 1, 2};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            bool gh;
-            g.yoff[k] = DIM > 1 ? (map1(y + ds[k], p.ny, p.bc_lo[1], p.bc_hi[1], gh) - y) * p.nx : 0;
-            g.zoff[k] = DIM > 2 ? (map1(z + ds[k], p.nz, p.bc_lo[2], p.bc_hi[2], gh) - z) * p.nx * p.ny : 0;
-        }
-    }
-    if constexpr (DIM == 3) {
-        g.sb[0] = 4u * unsigned(g.idx0 + g.oa);
-        g.sb[1] = 4u * unsigned(g.idx0);
-        g.sb[2] = 4u * unsigned(g.idx0 + g.oc);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            g.sb[3 + k] = 4u * unsigned(g.idx0 + g.yoff[k]);
-            g.sb[7 + k] = 4u * unsigned(g.idx0 + g.zoff[k]);
+            if constexpr (DIM > 1) io.y[k] = at(i0 + (map1(y + ds[k], p.ny, p.bc_lo[1], p.bc_hi[1]) - y) * nxe);
+            if constexpr (DIM > 2) io.z[k] = at(i0 + (map1(z + ds[k], p.nz, p.bc_lo[2], p.bc_hi[2]) - z) * nxe * p.ny);
         }
     }
     // threads per block as the launcher sets them (rlb_step_f32_launch.cuh), a
@@ -968,11 +1086,7 @@ __global__ void __launch_bounds__(32 * RLB_F32_BY, VEC2 ? RLB_F32_MINB : 1)
     // sit at fixed offsets from one base address
     constexpr int nthr = (DIM == 1 && !LIN) ? 128 : 32 * RLB_F32_BY;
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    constexpr bool STAGE = kStageOn && VEC2 && !EULER;
-    update_pair<DIM, EULER, VEC2, LD_NC, kParkOn, STAGE, NP, LAT, REC64>(p, g, p.f_eta_over_s, p.f_kbulk, f, h, fo, ho,
-                                                                  prev, ps,
-                                                         s_park + tid, nthr,
-                                                         s_park + (kParkOn ? kParkSlots * nthr : 0) + tid, nthr);
+    update_pair<EULER, (DIM > 1), NP, LAT, REC64>(p, io, has1, p.f_eta_over_s, s_park + tid, nthr);
 }
 
 }  // namespace f32

@@ -18,7 +18,7 @@ constexpr int kBulkThreads = 256;   // 32 x 8
 // the row and plane maps
 constexpr size_t bulk_smem_bytes()
 {
-    return sizeof(float) * size_t(kBulkBufs) * kTileFloats + sizeof(f2) * size_t(kParkSlots) * kBulkThreads +
+    return sizeof(float) * size_t(kBulkBufs) * kTileFloats + sizeof(f2) * size_t(kParkH + kEqSlots) * kBulkThreads +
            sizeof(unsigned long long) * kBulkBufs + 2 * sizeof(int) * kBulkBufs + sizeof(int) * 16;
 }
 
@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(kBulkThreads, 2)
     float *tiles = reinterpret_cast<float *>(smem);
     f2 *park = reinterpret_cast<f2 *>(smem + sizeof(float) * size_t(kBulkBufs) * kTileFloats);
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(
-        smem + sizeof(float) * size_t(kBulkBufs) * kTileFloats + sizeof(f2) * size_t(kParkSlots) * kBulkThreads);
+        smem + sizeof(float) * size_t(kBulkBufs) * kTileFloats + sizeof(f2) * size_t(kParkH + kEqSlots) * kBulkThreads);
     int *issued = reinterpret_cast<int *>(bars + kBulkBufs);
     int *done = issued + kBulkBufs;
     int *ymap = done + kBulkBufs, *zmap = ymap + 12;
@@ -86,23 +86,10 @@ __global__ void __launch_bounds__(kBulkThreads, 2)
     });
 
     const int x0 = b.x0t + 2 * tx, y = b.y0 + ty, z = b.z;
-    Geo g;
-    g.idx0 = x0 + p.nx * (y + p.ny * z);
-    g.x0 = x0;
-    g.has1 = true;
-    g.idx1 = g.idx0 + 1;
-    g.oa = 0;
-    g.oc = 0;
-    g.xfix = 0u;
-    if (x0 == 0) g.xfix |= p.bc_lo[0] == BC_OUTFLOW ? XF_LO_CLAMP : XF_LO_GHOST;
-    if (x0 + 2 >= p.nx) g.xfix |= p.bc_hi[0] == BC_OUTFLOW ? XF_HI_CLAMP : XF_HI_GHOST;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        g.yoff[k] = 0;   // the tile source takes neighbours by axis and distance
-        g.zoff[k] = 0;
-    }
-    update_pair<3, false, true, LD_NC, kParkOn, false, 19, LAT, false, true>(
-        p, g, p.f_eta_over_s, p.f_kbulk, f, h, fo, ho, prev, p.ps, park + tid, kBulkThreads, nullptr, 0, &b);
+    BulkIO<LAT> io{{p, f, h, fo, ho, prev, p.ps, x0 + p.nx * (y + p.ny * z), 0u, p.f_kbulk}, &b};
+    if (x0 == 0) io.xfix |= p.bc_lo[0] == BC_OUTFLOW ? XF_LO_CLAMP : XF_LO_GHOST;
+    if (x0 + 2 >= p.nx) io.xfix |= p.bc_hi[0] == BC_OUTFLOW ? XF_HI_CLAMP : XF_HI_GHOST;
+    update_pair<false, true, 19, LAT, false>(p, io, true, p.f_eta_over_s, park + tid, kBulkThreads);
 
     // after a timeout: let the copies this block issued land before the
     // shared memory is released (bounded as well)

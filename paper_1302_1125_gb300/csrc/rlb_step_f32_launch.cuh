@@ -22,15 +22,14 @@ inline bool f32_use_linear(const StepParams &p, int dim)
     return fill < 0.97;
 }
 
-template <int DIM, bool EULER, bool VEC2, int LAT, int NP, bool LIN, bool REC64 = false>
-cudaError_t launch_f32(const StepParams &p, const float *f, const float *h, float *fo, float *ho, float *prev,
-                       cudaStream_t s)
+template <int DIM, bool EULER, bool ODDP, int LAT, int NP, bool LIN, bool REC64 = false>
+cudaError_t launch_f32(const StepParams &p, const float *f, float *fo, float *prev, cudaStream_t s)
 {
     if constexpr (DIM == 2 && !EULER && NP == 19 && !REC64) {
-        if (p.sym == 2) return launch_f32<2, false, VEC2, LAT, 14, LIN>(p, f, h, fo, ho, prev, s);
+        if (p.sym == 2) return launch_f32<2, false, ODDP, LAT, 14, LIN>(p, f, fo, prev, s);
     }
     if constexpr (DIM == 1 && !EULER && NP == 19 && !LIN && !REC64) {
-        if (p.sym == 1) return launch_f32<1, false, VEC2, LAT, 7, false>(p, f, h, fo, ho, prev, s);
+        if (p.sym == 1) return launch_f32<1, false, ODDP, LAT, 7, false>(p, f, fo, prev, s);
     }
     const int npairs = (p.nx + 1) / 2;
     dim3 block, grid;
@@ -48,53 +47,55 @@ cudaError_t launch_f32(const StepParams &p, const float *f, const float *h, floa
         block = dim3(32, RLB_F32_BY, 1);
         grid = dim3((npairs + 31) / 32, (p.ny + RLB_F32_BY - 1) / RLB_F32_BY, p.nz);
     }
-    const size_t smem = f32::step_smem_bytes(int(block.x * block.y), f32::kStageOn && VEC2 && !EULER, DIM);
-    // the shared-memory limit is a per-device attribute of the kernel: set it
-    // once per device and instantiation (a repeated set is harmless, so the
-    // flags need no lock)
-    constexpr int kMaxDevices = 64;
-    static std::atomic<bool> attr_set[kMaxDevices];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= kMaxDevices || !attr_set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(f32::step_f32_kernel<DIM, EULER, VEC2, LAT, NP, LIN, REC64>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const size_t smem = EULER ? 0 : f32::park_bytes(int(block.x * block.y), DIM);
+    // above 48 KB the shared-memory limit is a per-device attribute of the
+    // kernel: set it once per device and instantiation (a repeated set is
+    // harmless, so the flags need no lock)
+    if (smem > 48 * 1024) {
+        constexpr int kMaxDevices = 64;
+        static std::atomic<bool> attr_set[kMaxDevices];
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
-        if (dev < kMaxDevices) attr_set[dev].store(true, std::memory_order_release);
+        if (dev >= kMaxDevices || !attr_set[dev].load(std::memory_order_acquire)) {
+            e = cudaFuncSetAttribute(f32::step_f32_kernel<DIM, EULER, ODDP, LAT, NP, LIN, REC64>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+            if (e != cudaSuccess) return e;
+            if (dev < kMaxDevices) attr_set[dev].store(true, std::memory_order_release);
+        }
     }
-    f32::step_f32_kernel<DIM, EULER, VEC2, LAT, NP, LIN, REC64><<<grid, block, smem, s>>>(p, f, h, fo, ho, prev);
+    f32::step_f32_kernel<DIM, EULER, ODDP, LAT, NP, LIN, REC64><<<grid, block, smem, s>>>(p, f, fo, prev);
     return cudaGetLastError();
 }
 
 // dim 2 or 3 (and 1 when !LIN), Euler or viscous, lattice from p.lat
 template <bool LIN>
-cudaError_t launch_f32_mapped(const StepParams &p, int dim, int euler, const float *f, const float *h, float *fo,
-                              float *ho, float *prev, cudaStream_t s)
+cudaError_t launch_f32_mapped(const StepParams &p, int dim, int euler, const float *f, float *fo, float *prev,
+                              cudaStream_t s)
 {
     auto go = [&](auto lc, auto ec, auto vc) -> cudaError_t {
         constexpr int L = decltype(lc)::value;
         constexpr bool E = decltype(ec)::value, V = decltype(vc)::value;
         if constexpr (!LIN) {
-            if (dim == 1) return launch_f32<1, E, V, L, 19, false>(p, f, h, fo, ho, prev, s);
+            if (dim == 1) return launch_f32<1, E, V, L, 19, false>(p, f, fo, prev, s);
         }
-        if (dim == 2) return launch_f32<2, E, V, L, 19, LIN>(p, f, h, fo, ho, prev, s);
-        return launch_f32<3, E, V, L, 19, LIN>(p, f, h, fo, ho, prev, s);
+        if (dim == 2) return launch_f32<2, E, V, L, 19, LIN>(p, f, fo, prev, s);
+        return launch_f32<3, E, V, L, 19, LIN>(p, f, fo, prev, s);
     };
-    // pair loads are 8-byte aligned when every row starts at an even index
-    const bool vec = p.nx % 2 == 0;
+    // periodic rows of odd length wrap to pairs that are not aligned
+    const bool oddp = p.nx % 2 != 0 && p.nx > 1 && (p.bc_lo[0] == BC_PERIODIC || p.bc_hi[0] == BC_PERIODIC);
     auto by_lat = [&](auto ec, auto vc) {
         return p.lat == 1 ? go(std::integral_constant<int, 1>{}, ec, vc)
                           : go(std::integral_constant<int, 0>{}, ec, vc);
     };
     auto by_vec = [&](auto ec) {
-        return vec ? by_lat(ec, std::true_type{}) : by_lat(ec, std::false_type{});
+        return oddp ? by_lat(ec, std::true_type{}) : by_lat(ec, std::false_type{});
     };
     return euler ? by_vec(std::true_type{}) : by_vec(std::false_type{});
 }
 
 // the linear instantiations (rlb_step_f32_lin.cu)
-cudaError_t launch_step_f32_linear(const StepParams &p, int dim, int euler, const float *f, const float *h,
-                                   float *fo, float *ho, float *prev, cudaStream_t s);
+cudaError_t launch_step_f32_linear(const StepParams &p, int dim, int euler, const float *f, float *fo, float *prev,
+                                   cudaStream_t s);
 
 }  // namespace rlb

@@ -5,10 +5,10 @@
 
 namespace rlb {
 
-cudaError_t launch_step_f32_linear(const StepParams &p, int dim, int euler, const float *f, const float *h,
-                                   float *fo, float *ho, float *prev, cudaStream_t s)
+cudaError_t launch_step_f32_linear(const StepParams &p, int dim, int euler, const float *f, float *fo, float *prev,
+                                   cudaStream_t s)
 {
-    return launch_f32_mapped<true>(p, dim, euler, f, h, fo, ho, prev, s);
+    return launch_f32_mapped<true>(p, dim, euler, f, fo, prev, s);
 }
 
 }  // namespace rlb

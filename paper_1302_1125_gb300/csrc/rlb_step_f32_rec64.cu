@@ -8,12 +8,12 @@
 
 namespace rlb {
 
-cudaError_t launch_step_f32_rec64(const StepParams &p, int dim, const float *f, const float *h, float *fo,
-                                  float *ho, float *prev, cudaStream_t s)
+cudaError_t launch_step_f32_rec64(const StepParams &p, int dim, const float *f, float *fo, float *prev,
+                                  cudaStream_t s)
 {
-    if (dim == 1) return launch_f32<1, false, true, 0, 19, false, true>(p, f, h, fo, ho, prev, s);
-    if (dim == 2) return launch_f32<2, false, true, 0, 19, false, true>(p, f, h, fo, ho, prev, s);
-    return launch_f32<3, false, true, 0, 19, false, true>(p, f, h, fo, ho, prev, s);
+    if (dim == 1) return launch_f32<1, false, false, 0, 19, false, true>(p, f, fo, prev, s);
+    if (dim == 2) return launch_f32<2, false, false, 0, 19, false, true>(p, f, fo, prev, s);
+    return launch_f32<3, false, false, 0, 19, false, true>(p, f, fo, prev, s);
 }
 
 }  // namespace rlb
