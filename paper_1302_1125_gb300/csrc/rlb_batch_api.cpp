@@ -50,6 +50,7 @@ struct rlb_batch {
     double *h_tot = nullptr;
     rlb_batch_tuning tune{};
     int nclusters = 0;               // clusters resident at once for `tune`
+    bool shape_set = false;          // the launch shape was set, tuned or chosen (choose_shape)
     bool plan_ok = false;
     std::vector<long long> plan_steps;
     cudaStream_t stream = nullptr, cap_stream = nullptr;
@@ -295,6 +296,49 @@ rlb_status apply_tuning(rlb_batch *b, const rlb_batch_tuning &t)
     return RLB_OK;
 }
 
+// The launch shape of a batch that nobody tuned, chosen at its first step
+// call: the one whose plan has the least critical path (rlb_batch_plan, in
+// passes) times the time of a pass.  A pass of a block costs more the more
+// warps share its SM, and a little more in a cluster (its barrier); the
+// costs are those measured on GB300 over batches of 16 to 512 tubes of 256 to
+// 8192 cells (us a pass: 256 threads 6.4-6.8, 384 8.1-9.2, 512 12.4 with
+// single blocks; 7.0-7.8, 8.3-10.2, 14.0 in clusters of 2; 8.1-8.5, 10-11,
+// 14.3-14.9 in clusters of 4 and 8; with 7 classes a little over half).
+// 512 tubes: 384 threads in clusters of 2, 25.6 ms where 256 threads in single
+// blocks take 59.9 ms.
+rlb_status choose_shape(rlb_batch *b, const long long *steps)
+{
+    b->shape_set = true;
+    const bool sym = b->opt.symmetry_1d != 0;
+    const double cost[3] = {sym ? 3.4 : 6.6, sym ? 4.2 : 8.8, sym ? 5.2 : 13.0};
+    const double join[4] = {1.0, sym ? 1.2 : 1.12, sym ? 1.35 : 1.2, sym ? 1.4 : 1.25};
+    // job capacities: one for large batches, whose plans take longer to make
+    // and whose tubes outnumber the clusters anyway
+    const bool large = b->B > 2048;
+    rlb_batch_tuning best = b->tune;
+    double best_cost = -1.0;
+    for (int i = 0; i < 3; ++i) {
+        for (int j = 0; j < 4; ++j) {
+            rlb_batch_tuning t{256 + 128 * i, 256 + 128 * i, 1 << j, 1, 0.0};
+            int n = 0;
+            if (rlb_status st = resident_clusters(b, t, n); st != RLB_OK) return st;
+            if (n < 1) continue;
+            for (int k = large ? 4 : 1; k <= 4; k *= 2) {
+                t.pairs_per_thread = k;
+                Plan pl;
+                std::string why;
+                if (make_plan(b->B, b->nx.data(), steps, t, n, pl, why) != RLB_OK) continue;
+                const double c = double(pl.critical) * cost[i] * join[j];
+                if (best_cost < 0.0 || c < best_cost) {
+                    best_cost = c;
+                    best = t;
+                }
+            }
+        }
+    }
+    return best_cost < 0.0 ? RLB_OK : apply_tuning(b, best);
+}
+
 rlb_status ensure_graph(rlb_batch *b)
 {
     if (b->graph) return RLB_OK;
@@ -519,8 +563,8 @@ rlb_status rlb_batch_create(int B, const int *nx, const double *eta_over_s, cons
     sp.f_kw = float(sp.kw);
     sp.f_tau_override = float(sp.tau_override);
 
-    // a default that fits every GB300 configuration; rlb_batch_autotune
-    // measures the alternatives
+    // a shape that fits every GB300 configuration, until the first step call
+    // chooses one for its step counts; rlb_batch_autotune measures them
     rlb_batch_tuning t{256, 256, 1, 1, 0.0};
     const rlb_status st = apply_tuning(b, t);
     if (st != RLB_OK) {
@@ -563,6 +607,7 @@ rlb_status rlb_batch_step(rlb_batch *b, const long long *nsteps)
     for (int i = 0; i < b->B; ++i) any = any || nsteps[i] > 0;
     if (!any) return RLB_OK;
     RLB_BCUDA(b, cudaSetDevice(b->device));
+    if (!b->shape_set && (st = choose_shape(b, nsteps)) != RLB_OK) return st;
     if ((st = prepare(b, nsteps)) != RLB_OK) return st;
     if ((st = ensure_graph(b)) != RLB_OK) return st;
     RLB_BCUDA(b, cudaGraphLaunch(b->graph, b->stream));
@@ -606,7 +651,9 @@ rlb_status rlb_batch_set_tuning(rlb_batch *b, const rlb_batch_tuning *t)
     if (!b) return bfail(nullptr, RLB_E_INVALID, "batch is NULL");
     if (!t) return bfail(b, RLB_E_INVALID, "tuning is NULL");
     RLB_BCUDA(b, cudaSetDevice(b->device));
-    return apply_tuning(b, *t);
+    const rlb_status st = apply_tuning(b, *t);
+    if (st == RLB_OK) b->shape_set = true;
+    return st;
 }
 
 rlb_status rlb_batch_get_tuning(const rlb_batch *b, rlb_batch_tuning *t, int *resident_clusters)
@@ -699,6 +746,7 @@ rlb_status rlb_batch_autotune(rlb_batch *b, const long long *nsteps, int divisor
     const rlb_batch_tuning chosen = done[k];
     st = apply_tuning(b, chosen);
     if (st != RLB_OK) return st;
+    b->shape_set = true;
     b->tune.ms = chosen.ms;
     if (n_trials) *n_trials = int(done.size());
     for (int i = 0; i < max_trials && i < int(done.size()); ++i) trials[i] = done[i];
