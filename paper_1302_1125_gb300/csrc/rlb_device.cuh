@@ -43,6 +43,18 @@ enum { ST_NONPHYSICAL = 1, ST_ASYMMETRIC = 2, ST_TIMEOUT = 4 };   // ST_ASYMMETR
                                                                  // reduction cannot take; ST_TIMEOUT: a bounded
                                                                  // wait of a kernel gave up
 
+// Consecutive steps overlap their launches (programmatic dependent launch,
+// launch_overlapped): a step's blocks may start while the step before runs,
+// and wait here, before their first access to global memory, until it has
+// finished and its writes are visible.  Only then may the next step start, so
+// at most two steps are in flight.  The populations are read with plain loads:
+// the read-only path requires data that no other kernel writes meanwhile.
+__device__ __forceinline__ void grid_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Macroscopic state and recovery (Sec. II: T^{0 mu} plus eps = 3P, Eq. 38)
 // ---------------------------------------------------------------------------
@@ -71,15 +83,45 @@ __host__ __device__ __forceinline__ bool recover(double E, double Mx, double My,
     return (E > 0.0) && (D > 0.0) && isfinite(m.n) && isfinite(s);
 }
 
+// The macroscopic state with gamma and 1 / gamma, and the same recovery with
+// the divisions and square roots that share a denominator done once (a
+// division is 8 to 10 operations of the FP64 pipe): 1/gamma by the reciprocal
+// square root, s = 1/(4 P gamma) and n from it.
+struct MacroG : Macro {
+    double g, ig;
+};
+__device__ __forceinline__ bool recover_g(double E, double Mx, double My, double Mz, double N0, MacroG &m)
+{
+    const double M2 = Mx * Mx + My * My + Mz * Mz;
+    const double D = E * E - M2;
+    m.P = D / (E + sqrt(4.0 * E * E - 3.0 * M2));
+    const double r = 1.0 / (4.0 * m.P);
+    const double g2 = (E + m.P) * r;
+    m.ig = rsqrt(g2);
+    m.g = g2 * m.ig;
+    const double s = r * m.ig;
+    m.ux = Mx * s;
+    m.uy = My * s;
+    m.uz = Mz * s;
+    m.n = N0 * m.ig;
+    return (E > 0.0) && (D > 0.0) && isfinite(m.n) && isfinite(s);
+}
+__device__ __forceinline__ void gamma_of(MacroG &m)
+{
+    const double w = 1.0 + (m.ux * m.ux + m.uy * m.uy + m.uz * m.uz);
+    m.ig = rsqrt(w);
+    m.g = w * m.ig;
+}
+
 // tau from eta/s (Eq. 41 with s = n (4 - ln lambda), lambda = n / n_eq,
 // n_eq = 16 T^3 / pi^2, T = P/n, Sec. III): tau = 1/2 + nu^2 (eta/s)(4 - ln lambda)/(4 T)
 template <int LAT = 0>
 __device__ __forceinline__ double tau_of(double P, double n, double eta_over_s)
 {
-    const double T = P / n;
-    const double lam = n * kPi2Over16 / (T * T * T);
+    const double b = n / P;   // 1 / T
+    const double lam = n * kPi2Over16 * (b * b * b);
     const double sfac = fmax(4.0 - log(lam), kSMin);
-    return 0.5 + Lat<LAT>::nu2 * eta_over_s * sfac / (4.0 * T);
+    return 0.5 + (0.25 * Lat<LAT>::nu2 * eta_over_s) * sfac * b;
 }
 
 // ---------------------------------------------------------------------------
@@ -137,6 +179,46 @@ __host__ __device__ __forceinline__ void coef_h(const Macro &m, Coef<double> &k)
     k.Ko[0] = 9.0 * B * ux * uy;
     k.Ko[1] = 9.0 * B * ux * uz;
     k.Ko[2] = 9.0 * B * uy * uz;
+}
+
+// The same coefficients from a state that carries gamma and 1/gamma; those of
+// h with u = u' / gamma multiplied out (n gamma u = n u')
+template <int LAT = 0>
+__device__ __forceinline__ void coef_f_g(const MacroG &m, Coef<double> &k)
+{
+    const double u2 = m.ux * m.ux + m.uy * m.uy + m.uz * m.uz;
+    const double A = m.P * Lat<LAT>::inv_sigma2;
+    const double b = A * Lat<LAT>::four_over_xi0 * m.g;
+    const double d = A * Lat<LAT>::a3f;
+    const double o = A * Lat<LAT>::a2f;
+    const double ox = o * m.ux;
+    k.K0 = A * (1.0 - (16.0 / 15.0) * u2);
+    k.Kb[0] = b * m.ux;
+    k.Kb[1] = b * m.uy;
+    k.Kb[2] = b * m.uz;
+    k.Kd[0] = d * m.ux * m.ux;
+    k.Kd[1] = d * m.uy * m.uy;
+    k.Kd[2] = d * m.uz * m.uz;
+    k.Ko[0] = ox * m.uy;
+    k.Ko[1] = ox * m.uz;
+    k.Ko[2] = o * m.uy * m.uz;
+}
+template <int LAT = 0>
+__device__ __forceinline__ void coef_h_g(const MacroG &m, Coef<double> &k)
+{
+    const double u2p = m.ux * m.ux + m.uy * m.uy + m.uz * m.uz;
+    const double t = m.n * m.ig;
+    const double b = 3.0 * m.n, d = 4.5 * t, o = 9.0 * t, ox = o * m.ux;
+    k.K0 = m.n * m.g * Lat<LAT>::c0ct - 1.5 * t * u2p;
+    k.Kb[0] = b * m.ux;
+    k.Kb[1] = b * m.uy;
+    k.Kb[2] = b * m.uz;
+    k.Kd[0] = d * m.ux * m.ux;
+    k.Kd[1] = d * m.uy * m.uy;
+    k.Kd[2] = d * m.uz * m.uz;
+    k.Ko[0] = ox * m.uy;
+    k.Ko[1] = ox * m.uz;
+    k.Ko[2] = o * m.uy * m.uz;
 }
 
 // An equilibrium with the lattice weights and the diagonal factors (2 and 4
@@ -221,6 +303,55 @@ __host__ __device__ __forceinline__ R eq_pop(const EqW<R> &e)
         v = (cb > 0) ? v + e.db[b] : v - e.db[b];
         v = (ca * cb > 0) ? v + e.dk[ko] : v - e.dk[ko];
         return v;
+    }
+}
+
+// The equilibrium with the sums its populations share formed once, so that a
+// population is one addition: per axis w1 (K0 + Kd) and w1 Kb; per plane (xy,
+// xz, yz) the even parts p = base + dk, m = base - dk and the odd parts s =
+// db_a + db_b, t = db_a - db_b (signs ++ p + s, +- m + t, -+ m - t, -- p - s).
+// 55 FP64 operations a distribution instead of 89.
+struct EqP {
+    double r0, ax[3], ab[3], p[3], m[3], s[3], t[3];
+};
+template <int DM>
+__device__ __forceinline__ EqP fold(const Coef<double> &k, double w0, double w1, double w2)
+{
+    EqP e;
+    e.r0 = w0 * k.K0;
+    double db[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        e.ax[j] = w1 * (k.K0 + k.Kd[j]);
+        e.ab[j] = w1 * k.Kb[j];
+        db[j] = (double(DM) * w2) * k.Kb[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int a = j == 2 ? 1 : 0, b = j == 0 ? 1 : 2;
+        const double base = w2 * (k.K0 + double(DM * DM) * (k.Kd[a] + k.Kd[b]));
+        const double dk = (double(DM * DM) * w2) * k.Ko[j];
+        e.p[j] = base + dk;
+        e.m[j] = base - dk;
+        e.s[j] = db[a] + db[b];
+        e.t[j] = db[a] - db[b];
+    }
+    return e;
+}
+template <int I>
+__device__ __forceinline__ double eq_pop(const EqP &e)
+{
+    constexpr int cx = cdir<I, 0>(), cy = cdir<I, 1>(), cz = cdir<I, 2>();
+    if constexpr (shell<I>() == 0) {
+        return e.r0;
+    } else if constexpr (shell<I>() == 1) {
+        constexpr int a = cx != 0 ? 0 : (cy != 0 ? 1 : 2);
+        return cx + cy + cz > 0 ? e.ax[a] + e.ab[a] : e.ax[a] - e.ab[a];
+    } else {
+        constexpr int ca = cx != 0 ? cx : cy, cb = cz != 0 ? cz : cy;
+        constexpr int j = cz == 0 ? 0 : (cx != 0 ? 1 : 2);
+        if constexpr (ca > 0) return cb > 0 ? e.p[j] + e.s[j] : e.m[j] + e.t[j];
+        else return cb > 0 ? e.m[j] - e.t[j] : e.p[j] - e.s[j];
     }
 }
 

@@ -32,6 +32,24 @@ struct StepParams {
     float f_ghost_f[19], f_ghost_h[19];
 };
 
+// launch a kernel that calls grid_wait (rlb_device.cuh) so that it may start
+// while the kernel before it on the stream still runs
+template <typename... P, typename... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Storage of a grid's populations: planes of stride ps (FP64 form; FP32 grids
 // staged by bulk copies), or blocks of 32 cells (the other FP32 grids,
 // rlb_step_f32.cuh)

@@ -546,7 +546,7 @@ struct BlockIO {
     static __device__ __forceinline__ f2 ld(const char *q)
     {
         f2 v;
-        asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2+%3];" : "=f"(v.x), "=f"(v.y) : "l"(q), "n"(K * kBlk * 4));
+        asm volatile("ld.global.v2.f32 {%0, %1}, [%2+%3];" : "=f"(v.x), "=f"(v.y) : "l"(q), "n"(K * kBlk * 4));
         return v;
     }
     template <int J>
@@ -560,7 +560,8 @@ struct BlockIO {
             s.v[2] = ld<T::K>(r);
             if constexpr (ODDP) {
                 s.ex = 0.0f;
-                if (xfix & (XF_LO_EX | XF_HI_EX)) s.ex = __ldg(reinterpret_cast<const float *>(e) + T::K * kBlk);
+                if (xfix & (XF_LO_EX | XF_HI_EX))
+                    asm volatile("ld.global.f32 %0, [%1+%2];" : "=f"(s.ex) : "l"(e), "n"(T::K * kBlk * 4));
             }
         }
         s.v[1] = ld<T::K>(c);
@@ -593,8 +594,7 @@ struct BlockIO {
     template <int J>
     __device__ __forceinline__ f2 own() const
     {
-        const float2 v = __ldg(reinterpret_cast<const float2 *>(c + Item<NP, J>::K * kBlk * 4));
-        return f2{v.x, v.y};
+        return ld<Item<NP, J>::K>(c);
     }
     template <int S, int J>
     __device__ __forceinline__ f2 pre()
@@ -1081,6 +1081,7 @@ __global__ void __launch_bounds__(32 * RLB_F32_BY, RLB_F32_MINB)
             if constexpr (DIM > 2) io.z[k] = at(i0 + (map1(z + ds[k], p.nz, p.bc_lo[2], p.bc_hi[2]) - z) * nxe * p.ny);
         }
     }
+    grid_wait();
     // threads per block as the launcher sets them (rlb_step_f32_launch.cuh), a
     // compile-time constant so that the shared-memory slots of this thread
     // sit at fixed offsets from one base address

@@ -64,8 +64,8 @@ cudaError_t launch_f32(const StepParams &p, const float *f, float *fo, float *pr
             if (dev < kMaxDevices) attr_set[dev].store(true, std::memory_order_release);
         }
     }
-    f32::step_f32_kernel<DIM, EULER, ODDP, LAT, NP, LIN, REC64><<<grid, block, smem, s>>>(p, f, fo, prev);
-    return cudaGetLastError();
+    return launch_overlapped(f32::step_f32_kernel<DIM, EULER, ODDP, LAT, NP, LIN, REC64>, grid, block, smem, s, p, f, fo,
+                             prev);
 }
 
 // dim 2 or 3 (and 1 when !LIN), Euler or viscous, lattice from p.lat
