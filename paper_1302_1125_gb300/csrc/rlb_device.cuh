@@ -83,6 +83,10 @@ __host__ __device__ __forceinline__ bool recover(double E, double Mx, double My,
     return (E > 0.0) && (D > 0.0) && isfinite(m.n) && isfinite(s);
 }
 
+// The FP64 step rounds alike in both of its kernels (rlb_kernels.cuh): what
+// follows states its fused operations, so that none is left to the compiler.
+__device__ __forceinline__ double sq3(double x, double y, double z) { return fma(z, z, fma(y, y, x * x)); }
+
 // The macroscopic state with gamma and 1 / gamma, and the same recovery with
 // the divisions and square roots that share a denominator done once (a
 // division is 8 to 10 operations of the FP64 pipe): 1/gamma by the reciprocal
@@ -92,9 +96,9 @@ struct MacroG : Macro {
 };
 __device__ __forceinline__ bool recover_g(double E, double Mx, double My, double Mz, double N0, MacroG &m)
 {
-    const double M2 = Mx * Mx + My * My + Mz * Mz;
-    const double D = E * E - M2;
-    m.P = D / (E + sqrt(4.0 * E * E - 3.0 * M2));
+    const double M2 = sq3(Mx, My, Mz);
+    const double D = fma(E, E, -M2);
+    m.P = D / (E + sqrt(fma(4.0 * E, E, -3.0 * M2)));
     const double r = 1.0 / (4.0 * m.P);
     const double g2 = (E + m.P) * r;
     m.ig = rsqrt(g2);
@@ -108,7 +112,7 @@ __device__ __forceinline__ bool recover_g(double E, double Mx, double My, double
 }
 __device__ __forceinline__ void gamma_of(MacroG &m)
 {
-    const double w = 1.0 + (m.ux * m.ux + m.uy * m.uy + m.uz * m.uz);
+    const double w = 1.0 + sq3(m.ux, m.uy, m.uz);
     m.ig = rsqrt(w);
     m.g = w * m.ig;
 }
@@ -121,7 +125,7 @@ __device__ __forceinline__ double tau_of(double P, double n, double eta_over_s)
     const double b = n / P;   // 1 / T
     const double lam = n * kPi2Over16 * (b * b * b);
     const double sfac = fmax(4.0 - log(lam), kSMin);
-    return 0.5 + (0.25 * Lat<LAT>::nu2 * eta_over_s) * sfac * b;
+    return fma((0.25 * Lat<LAT>::nu2 * eta_over_s) * sfac, b, 0.5);
 }
 
 // ---------------------------------------------------------------------------
@@ -186,13 +190,13 @@ __host__ __device__ __forceinline__ void coef_h(const Macro &m, Coef<double> &k)
 template <int LAT = 0>
 __device__ __forceinline__ void coef_f_g(const MacroG &m, Coef<double> &k)
 {
-    const double u2 = m.ux * m.ux + m.uy * m.uy + m.uz * m.uz;
+    const double u2 = sq3(m.ux, m.uy, m.uz);
     const double A = m.P * Lat<LAT>::inv_sigma2;
     const double b = A * Lat<LAT>::four_over_xi0 * m.g;
     const double d = A * Lat<LAT>::a3f;
     const double o = A * Lat<LAT>::a2f;
     const double ox = o * m.ux;
-    k.K0 = A * (1.0 - (16.0 / 15.0) * u2);
+    k.K0 = A * fma(-16.0 / 15.0, u2, 1.0);
     k.Kb[0] = b * m.ux;
     k.Kb[1] = b * m.uy;
     k.Kb[2] = b * m.uz;
@@ -206,10 +210,10 @@ __device__ __forceinline__ void coef_f_g(const MacroG &m, Coef<double> &k)
 template <int LAT = 0>
 __device__ __forceinline__ void coef_h_g(const MacroG &m, Coef<double> &k)
 {
-    const double u2p = m.ux * m.ux + m.uy * m.uy + m.uz * m.uz;
+    const double u2p = sq3(m.ux, m.uy, m.uz);
     const double t = m.n * m.ig;
     const double b = 3.0 * m.n, d = 4.5 * t, o = 9.0 * t, ox = o * m.ux;
-    k.K0 = m.n * m.g * Lat<LAT>::c0ct - 1.5 * t * u2p;
+    k.K0 = fma(m.n * m.g, Lat<LAT>::c0ct, -1.5 * t * u2p);
     k.Kb[0] = b * m.ux;
     k.Kb[1] = b * m.uy;
     k.Kb[2] = b * m.uz;
@@ -269,12 +273,12 @@ __host__ __device__ __forceinline__ Coef<double> extrapolate(const Coef<double> 
                                                              const Coef<double> &b)
 {
     Coef<double> k;
-    k.K0 = 2.0 * a.K0 - b.K0;
+    k.K0 = fma(2.0, a.K0, -b.K0);   // explicit: the same rounding wherever a and b come from
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        k.Kb[j] = 2.0 * a.Kb[j] - b.Kb[j];
-        k.Kd[j] = 2.0 * a.Kd[j] - b.Kd[j];
-        k.Ko[j] = 2.0 * a.Ko[j] - b.Ko[j];
+        k.Kb[j] = fma(2.0, a.Kb[j], -b.Kb[j]);
+        k.Kd[j] = fma(2.0, a.Kd[j], -b.Kd[j]);
+        k.Ko[j] = fma(2.0, a.Ko[j], -b.Ko[j]);
     }
     return k;
 }
@@ -317,22 +321,23 @@ struct EqP {
 template <int DM>
 __device__ __forceinline__ EqP fold(const Coef<double> &k, double w0, double w1, double w2)
 {
+    // (single roundings here, not fused into the sums that use them, so that
+    // both step kernels round alike)
     EqP e;
-    e.r0 = w0 * k.K0;
+    e.r0 = __dmul_rn(w0, k.K0);
     double db[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        e.ax[j] = w1 * (k.K0 + k.Kd[j]);
-        e.ab[j] = w1 * k.Kb[j];
-        db[j] = (double(DM) * w2) * k.Kb[j];
+        e.ax[j] = __dmul_rn(w1, k.K0 + k.Kd[j]);
+        e.ab[j] = __dmul_rn(w1, k.Kb[j]);
+        db[j] = __dmul_rn(double(DM) * w2, k.Kb[j]);
     }
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         const int a = j == 2 ? 1 : 0, b = j == 0 ? 1 : 2;
-        const double base = w2 * (k.K0 + double(DM * DM) * (k.Kd[a] + k.Kd[b]));
-        const double dk = (double(DM * DM) * w2) * k.Ko[j];
-        e.p[j] = base + dk;
-        e.m[j] = base - dk;
+        const double base = __dmul_rn(w2, fma(double(DM * DM), k.Kd[a] + k.Kd[b], k.K0));
+        e.p[j] = fma(double(DM * DM) * w2, k.Ko[j], base);
+        e.m[j] = fma(-double(DM * DM) * w2, k.Ko[j], base);
         e.s[j] = db[a] + db[b];
         e.t[j] = db[a] - db[b];
     }

@@ -25,36 +25,39 @@ cudaError_t launch_step_np(const StepParams &p, const T *f, const T *h, T *fo, T
                           cudaStream_t s)
 {
     const long long cells = (long long)p.nx * p.ny * p.nz;
-    // Grids with fewer cells than one block of 128 per SM: blocks of one to
-    // four warps of consecutive cells (x-fastest order) spread the cells over
-    // more SMs.  Measured: steps 6 % shorter on 800- to 8192-cell tubes and
-    // 32 x 16 x 16 grids.  The step time of such grids stays set by one
-    // warp's FP64 instructions at one scheduler's FP64 rate.
+    // Grids with fewer cells than one block of 128 per SM: four warps to 32
+    // cells (step_split_kernel); in Euler mode blocks of one to four warps of
+    // consecutive cells (x-fastest order) spread the cells over more SMs.
     const int nsm = sm_count();
     if (cells < 128LL * nsm && p.mapping != 1 && p.mapping != 3) {   // 3: tiles (FP32: bulk-staged)
-        int bs = int(((cells + nsm - 1) / nsm + 31) / 32 * 32);
-        bs = bs < 32 ? 32 : (bs > 128 ? 128 : bs);
-        const unsigned nb = unsigned((cells + bs - 1) / bs);
-        if constexpr (DIM == 1) step_kernel<T, DIM, EULER, LAT, false, NP><<<nb, bs, 0, s>>>(p, f, h, fo, ho, prev);
-        else step_kernel<T, DIM, EULER, LAT, true, NP><<<nb, bs, 0, s>>>(p, f, h, fo, ho, prev);
-        return cudaGetLastError();
+        if constexpr (!EULER) {
+            return launch_overlapped(step_split_kernel<DIM, LAT, NP>, unsigned((cells + 31) / 32), dim3(32, 4, 1), 0, s, p,
+                                     f, h, fo, ho, prev);
+        } else {
+            int bs = int(((cells + nsm - 1) / nsm + 31) / 32 * 32);
+            bs = bs < 32 ? 32 : (bs > 128 ? 128 : bs);
+            const unsigned nb = unsigned((cells + bs - 1) / bs);
+            if constexpr (DIM == 1) return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP>, nb, bs, 0, s, p, f, h, fo, ho, prev);
+            else return launch_overlapped(step_kernel<T, DIM, EULER, LAT, true, NP>, nb, bs, 0, s, p, f, h, fo, ho, prev);
+        }
     }
     if constexpr (DIM == 1) {
-        step_kernel<T, DIM, EULER, LAT, false, NP><<<(p.nx + 127) / 128, 128, 0, s>>>(p, f, h, fo, ho, prev);
+        return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP>, (p.nx + 127) / 128, 128, 0, s, p, f, h, fo, ho,
+                                 prev);
     } else {
         // tiles of 32 x 4 cells when nx and ny fill them, else 128 consecutive
         // cells of the x-fastest order per block
         const long long tiles_x = (p.nx + 31) / 32, tiles_y = (p.ny + 3) / 4;
         const double fill = double(p.nx) * p.ny / double(tiles_x * 32 * tiles_y * 4);
         if (p.mapping == 2 || (p.mapping == 0 && fill < 0.97)) {
-            step_kernel<T, DIM, EULER, LAT, true, NP><<<unsigned((cells + 127) / 128), 128, 0, s>>>(p, f, h, fo, ho,
-                                                                                                    prev);
+            return launch_overlapped(step_kernel<T, DIM, EULER, LAT, true, NP>, unsigned((cells + 127) / 128), 128, 0, s,
+                                     p, f, h, fo, ho, prev);
         } else {
             const dim3 grid(unsigned(tiles_x), unsigned(tiles_y), p.nz);
-            step_kernel<T, DIM, EULER, LAT, false, NP><<<grid, dim3(32, 4, 1), 0, s>>>(p, f, h, fo, ho, prev);
+            return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP>, grid, dim3(32, 4, 1), 0, s, p, f, h, fo,
+                                     ho, prev);
         }
     }
-    return cudaGetLastError();
 }
 
 // the symmetry reductions (p.sym: 1 on 1-D grids, 2 on 2-D grids; viscous)
