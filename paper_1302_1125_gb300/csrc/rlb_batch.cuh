@@ -39,43 +39,38 @@ __device__ __forceinline__ void cluster_barrier()
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// geometry of the pair (x0, x0 + 1) of a tube of nx cells stored at `off`
-// (zero-gradient at both ends; an odd tube's last pair holds one pad cell)
-__device__ __forceinline__ f32::Geo tube_geo(int off, int nx, int x0)
+// the x stencil of the pair (x0, x0 + 1) of a tube of nx cells stored at `off`
+// (zero-gradient at both ends; an odd tube's last pair holds one pad cell):
+// distances of the pairs it takes for x0-2 and x0+2, and the fix-ups
+__device__ __forceinline__ void tube_ends(int nx, int x0, int &ol, int &orr, unsigned &xfix)
 {
-    f32::Geo g;
-    g.x0 = x0;
-    g.idx0 = off + x0;
-    g.has1 = x0 + 1 < nx;
-    g.oa = -2;
-    g.oc = 2;
-    g.xfix = 0u;
+    ol = -2;
+    orr = 2;
+    xfix = 0u;
     if (x0 == 0) {
-        g.oa = 0;
-        g.xfix |= f32::XF_LO_CLAMP;
+        ol = 0;
+        xfix |= f32::XF_LO_CLAMP;
     }
     if (x0 + 2 >= nx) {
-        g.oc = 0;
-        g.xfix |= g.has1 ? f32::XF_HI_CLAMP : f32::XF_HI_ODD1;
+        orr = 0;
+        xfix |= x0 + 1 < nx ? f32::XF_HI_CLAMP : f32::XF_HI_ODD1;
     } else if (x0 + 3 == nx) {
-        g.xfix |= f32::XF_HI_ODD3;
+        xfix |= f32::XF_HI_ODD3;
     }
-    return g;
 }
 
-// LD = f32::LD_CA for C = 1 (only this block writes the job's tubes),
-// f32::LD_CG for C > 1 (the other blocks of the cluster write them too).
-// The stencils are staged through shared memory by cp.async (see
-// update_pair).
+// Populations in blocks of 32 cells and stencils straight into registers, as
+// on grids (f32::BlockIO); plain loads, which after the block or cluster
+// barrier see what the other threads of the cluster wrote in the step before.
 // MAXT = launch bound: 512 caps the kernel at 128 registers (some spill),
 // 384 at 168, 256 leaves it unconstrained; the autotuner picks.
-template <int LD, int MAXT, int NP>
+template <int MAXT, int NP>
 __global__ void __launch_bounds__(MAXT, 1) tubes_kernel(const Args a)
 {
     __shared__ int s_off[kMaxJobTubes], s_nx[kMaxJobTubes], s_steps[kMaxJobTubes], s_par[kMaxJobTubes];
     __shared__ int s_tube[kMaxJobTubes], s_p0[kMaxJobTubes + 1];
     __shared__ float s_eos[kMaxJobTubes], s_kb[kMaxJobTubes];
-    extern __shared__ f2 s_dyn[];   // parked coefficients and staged stencils (see update_pair)
+    extern __shared__ f2 s_dyn[];   // parked coefficients (see update_pair)
 
     const int C = a.cluster;
     const unsigned rank = C > 1 ? cluster_rank() : 0u;
@@ -114,16 +109,24 @@ __global__ void __launch_bounds__(MAXT, 1) tubes_kernel(const Args a)
                 int i = 0;
                 while (i + 1 < J.count && q >= s_p0[i + 1]) ++i;
                 if (s < s_steps[i]) {
-                    const f32::Geo g = tube_geo(s_off[i], s_nx[i], 2 * (q - s_p0[i]));
+                    const int x0 = 2 * (q - s_p0[i]), i0 = s_off[i] + x0, nx = s_nx[i];
                     const bool odd = ((s_par[i] + s) & 1) != 0;
-                    const float *f = odd ? a.f1 : a.f0, *h = odd ? a.h1 : a.h0;
-                    float *fo = odd ? a.f0 : a.f1, *ho = odd ? a.h0 : a.h1;
-                    // the slots of the shared-memory arrays are MAXT apart (the
+                    const char *src = reinterpret_cast<const char *>(odd ? a.f1 : a.f0);
+                    char *dst = reinterpret_cast<char *>(odd ? a.f0 : a.f1);
+                    auto at = [](int k) { return sizeof(float) * f32::blk_at(k); };
+                    f32::BlockIO<1, false, NP, 0, false> io{a.p};
+                    int ol, orr;
+                    tube_ends(nx, x0, ol, orr, io.xfix);
+                    io.c = src + at(i0);
+                    io.l = src + at(i0 + ol);
+                    io.r = src + at(i0 + orr);
+                    io.o = dst + at(i0);
+                    io.pv = a.prev + f32::blk_prev_at(i0);
+                    io.kb = s_kb[i];
+                    // the slots of the shared-memory array are MAXT apart (the
                     // launch bound, a compile-time constant: fixed offsets
                     // from one base address), whatever blockDim.x <= MAXT is
-                    f32::StageIO<NP, LD> io{{a.p, f, h, fo, ho, a.prev, a.ps, g.idx0, g.xfix, s_kb[i]},
-                                            g.oa, g.oc, s_dyn + f32::kParkH * MAXT + threadIdx.x, MAXT, 0u};
-                    f32::update_pair<false, false, NP, 0, false>(a.p, io, g.has1, s_eos[i], s_dyn + threadIdx.x, MAXT);
+                    f32::update_pair<false, false, NP, 0, false>(a.p, io, x0 + 1 < nx, s_eos[i], s_dyn + threadIdx.x, MAXT);
                 }
             }
             if (C > 1) cluster_barrier();
@@ -134,14 +137,14 @@ __global__ void __launch_bounds__(MAXT, 1) tubes_kernel(const Args a)
     }
 }
 
-template <int LD, int MAXT, int NP>
+template <int MAXT, int NP>
 cudaError_t launch_variant(const Args &a, int threads, int cluster, cudaStream_t s, int *nclusters_out)
 {
-    auto kern = tubes_kernel<LD, MAXT, NP>;
+    auto kern = tubes_kernel<MAXT, NP>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nclusters_out ? unsigned(cluster) : unsigned(a.nclusters * cluster), 1, 1);
     cfg.blockDim = dim3(unsigned(threads), 1, 1);
-    const size_t smem = f32::tube_smem_bytes(MAXT);   // slots MAXT apart
+    const size_t smem = f32::park_bytes(MAXT, 1);   // slots MAXT apart
     cfg.dynamicSmemBytes = smem;
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
@@ -169,19 +172,13 @@ cudaError_t launch_variant(const Args &a, int threads, int cluster, cudaStream_t
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-template <int LD>
-cudaError_t launch_ld(const Args &a, int threads, int bound, int cluster, cudaStream_t s, int *nclusters_out)
+template <int NP>
+cudaError_t launch_np(const Args &a, int threads, int bound, int cluster, cudaStream_t s, int *nclusters_out)
 {
     if (threads < 32 || threads > bound || threads % 32 != 0) return cudaErrorInvalidValue;
-    if (a.np == 7) {
-        if (bound == 256) return launch_variant<LD, 256, 7>(a, threads, cluster, s, nclusters_out);
-        if (bound == 384) return launch_variant<LD, 384, 7>(a, threads, cluster, s, nclusters_out);
-        if (bound == 512) return launch_variant<LD, 512, 7>(a, threads, cluster, s, nclusters_out);
-        return cudaErrorInvalidValue;
-    }
-    if (bound == 256) return launch_variant<LD, 256, 19>(a, threads, cluster, s, nclusters_out);
-    if (bound == 384) return launch_variant<LD, 384, 19>(a, threads, cluster, s, nclusters_out);
-    if (bound == 512) return launch_variant<LD, 512, 19>(a, threads, cluster, s, nclusters_out);
+    if (bound == 256) return launch_variant<256, NP>(a, threads, cluster, s, nclusters_out);
+    if (bound == 384) return launch_variant<384, NP>(a, threads, cluster, s, nclusters_out);
+    if (bound == 512) return launch_variant<512, NP>(a, threads, cluster, s, nclusters_out);
     return cudaErrorInvalidValue;
 }
 

@@ -34,7 +34,7 @@ struct rlb_batch {
     int max_nx = 0;
     int max_clusters = 0;            // capacity of the cluster table
     void *block = nullptr;
-    float *f0 = nullptr, *h0 = nullptr, *f1 = nullptr, *h1 = nullptr, *prev = nullptr;
+    float *f0 = nullptr, *f1 = nullptr, *prev = nullptr;   // blocks of 32 cells, 38 populations (f, h) or 5 values each
     size_t state_bytes = 0;          // f0 .. prev, contiguous from f0
     double *stage = nullptr;         // 6 x total doubles
     Tube *d_tubes = nullptr;
@@ -219,11 +219,8 @@ rlb::batch::Args make_args(rlb_batch *b)
     a.cluster = b->tune.cluster;
     a.np = b->opt.symmetry_1d ? 7 : 19;
     a.f0 = b->f0;
-    a.h0 = b->h0;
     a.f1 = b->f1;
-    a.h1 = b->h1;
     a.prev = b->prev;
-    a.ps = b->ps;
     return a;
 }
 
@@ -298,37 +295,36 @@ rlb_status apply_tuning(rlb_batch *b, const rlb_batch_tuning &t)
 
 // The launch shape of a batch that nobody tuned, chosen at its first step
 // call: the one whose plan has the least critical path (rlb_batch_plan, in
-// passes) times the time of a pass.  A pass of a block costs more the more
-// warps share its SM, and a little more in a cluster (its barrier); the
-// costs are those measured on GB300 over batches of 16 to 512 tubes of 256 to
-// 8192 cells (us a pass: 256 threads 6.4-6.8, 384 8.1-9.2, 512 12.4 with
-// single blocks; 7.0-7.8, 8.3-10.2, 14.0 in clusters of 2; 8.1-8.5, 10-11,
-// 14.3-14.9 in clusters of 4 and 8; with 7 classes a little over half).
-// 512 tubes: 384 threads in clusters of 2, 25.6 ms where 256 threads in single
-// blocks take 59.9 ms.
+// passes) times the time of a pass.  A pass costs more the more threads share
+// the SM; the line below fits the autotuner's times on GB300 over batches of
+// 16 to 512 tubes of 256 to 8192 cells (us a pass with 128 / 256 / 384 / 512
+// threads an SM: 5.0-5.3, 5.6-6.5, 6.9-8.3, 9.2-9.9; with 7 classes 2.5-2.9,
+// 3.2-3.5, 4.0-4.2, 4.7-5.1), a cluster's barrier a few per cent more.
 rlb_status choose_shape(rlb_batch *b, const long long *steps)
 {
     b->shape_set = true;
     const bool sym = b->opt.symmetry_1d != 0;
-    const double cost[3] = {sym ? 3.4 : 6.6, sym ? 4.2 : 8.8, sym ? 5.2 : 13.0};
-    const double join[4] = {1.0, sym ? 1.2 : 1.12, sym ? 1.35 : 1.2, sym ? 1.4 : 1.25};
+    const double base = sym ? 2.2 : 3.9, per_thread = sym ? 0.0052 : 0.0108;
+    const double join[4] = {1.0, 1.03, 1.04, 1.06};
     // job capacities: one for large batches, whose plans take longer to make
     // and whose tubes outnumber the clusters anyway
     const bool large = b->B > 2048;
     rlb_batch_tuning best = b->tune;
     double best_cost = -1.0;
-    for (int i = 0; i < 3; ++i) {
+    for (int threads : {128, 256, 384, 512}) {
         for (int j = 0; j < 4; ++j) {
-            rlb_batch_tuning t{256 + 128 * i, 256 + 128 * i, 1 << j, 1, 0.0};
+            // small blocks in the 128-register variant, of which an SM holds several
+            rlb_batch_tuning t{threads, threads < 384 ? 512 : threads, 1 << j, 1, 0.0};
             int n = 0;
             if (rlb_status st = resident_clusters(b, t, n); st != RLB_OK) return st;
             if (n < 1) continue;
+            const double on_sm = double(threads) * double(n) * t.cluster / b->sms;
             for (int k = large ? 4 : 1; k <= 4; k *= 2) {
                 t.pairs_per_thread = k;
                 Plan pl;
                 std::string why;
                 if (make_plan(b->B, b->nx.data(), steps, t, n, pl, why) != RLB_OK) continue;
-                const double c = double(pl.critical) * cost[i] * join[j];
+                const double c = double(pl.critical) * (base + per_thread * on_sm) * join[j];
                 if (best_cost < 0.0 || c < best_cost) {
                     best_cost = c;
                     best = t;
@@ -375,8 +371,8 @@ rlb_status check_steps(rlb_batch *b, const long long *nsteps)
 rlb_status expand(rlb_batch *b)
 {
     if (!b->opt.symmetry_1d) return RLB_OK;
-    RLB_BCUDA(b, rlb::batch::launch_tubes_expand(b->B, b->max_nx, b->d_tubes, b->d_par, b->ps, b->f0, b->h0, b->f1,
-                                                 b->h1, b->stream));
+    RLB_BCUDA(b, rlb::batch::launch_tubes_expand(b->B, b->max_nx, b->d_tubes, b->d_par, b->f0, b->f1,
+                                                 b->stream));
     b->launches += 1;
     return RLB_OK;
 }
@@ -478,10 +474,8 @@ rlb_status rlb_batch_create(int B, const int *nx, const double *eta_over_s, cons
 
     const size_t plane = size_t(b->ps) * sizeof(float);
     size_t offs[14], o2 = 0;
-    offs[0] = o2; o2 += 19 * plane;                                   // f0
-    offs[1] = o2; o2 += 19 * plane;                                   // h0
-    offs[2] = o2; o2 += 19 * plane;                                   // f1
-    offs[3] = o2; o2 += 19 * plane;                                   // h1
+    offs[0] = o2; o2 += 38 * plane;                                   // f0, h0
+    offs[2] = o2; o2 += 38 * plane;                                   // f1, h1
     offs[4] = o2; o2 += 5 * plane;                                    // prev
     b->state_bytes = o2;
     o2 = aup(o2, 256);
@@ -501,9 +495,7 @@ rlb_status rlb_batch_create(int B, const int *nx, const double *eta_over_s, cons
     }
     char *base = (char *)b->block;
     b->f0 = (float *)(base + offs[0]);
-    b->h0 = (float *)(base + offs[1]);
     b->f1 = (float *)(base + offs[2]);
-    b->h1 = (float *)(base + offs[3]);
     b->prev = (float *)(base + offs[4]);
     b->d_par = (int *)(base + offs[5]);
     b->stage = (double *)(base + offs[6]);
@@ -591,8 +583,8 @@ rlb_status rlb_batch_init(rlb_batch *b, const double *n, const double *T, const 
         }
     }
     RLB_BCUDA(b, cudaMemsetAsync(b->d_par, 0, sizeof(int) * b->B, b->stream));
-    RLB_BCUDA(b, rlb::batch::launch_tubes_init(b->B, b->max_nx, b->d_tubes, b->d_pack, b->ps, dev[0], dev[1], dev[2],
-                                               b->f0, b->h0, b->prev, b->d_status, b->stream));
+    RLB_BCUDA(b, rlb::batch::launch_tubes_init(b->B, b->max_nx, b->d_tubes, b->d_pack, dev[0], dev[1], dev[2], b->f0,
+                                               b->prev, b->d_status, b->stream));
     b->launches += 1;
     const rlb_status st = check_status(b);
     return st == RLB_E_NONPHYSICAL ? bfail(b, RLB_E_INVALID, "initial state has n <= 0, T <= 0 or |u| >= 1") : st;
@@ -622,8 +614,8 @@ rlb_status rlb_batch_macroscopic(rlb_batch *b, double *out, int on_device)
     RLB_BCUDA(b, cudaSetDevice(b->device));
     if (rlb_status st = expand(b); st != RLB_OK) return st;
     double *dst = on_device ? out : b->stage;
-    RLB_BCUDA(b, rlb::batch::launch_tubes_macro(b->B, b->max_nx, b->d_tubes, b->d_pack, b->d_par, b->ps, b->total,
-                                                b->f0, b->h0, b->f1, b->h1, dst, b->d_status, b->stream));
+    RLB_BCUDA(b, rlb::batch::launch_tubes_macro(b->B, b->max_nx, b->d_tubes, b->d_pack, b->d_par, b->total, b->f0,
+                                                b->f1, dst, b->d_status, b->stream));
     b->launches += 1;
     if (!on_device)
         RLB_BCUDA(b, cudaMemcpyAsync(out, b->stage, 6 * sizeof(double) * size_t(b->total), cudaMemcpyDeviceToHost,
@@ -637,7 +629,7 @@ rlb_status rlb_batch_totals(rlb_batch *b, double *out)
     if (!out) return bfail(b, RLB_E_INVALID, "out is NULL");
     RLB_BCUDA(b, cudaSetDevice(b->device));
     if (rlb_status st = expand(b); st != RLB_OK) return st;
-    RLB_BCUDA(b, rlb::batch::launch_tubes_totals(b->B, b->d_tubes, b->d_par, b->ps, b->f0, b->h0, b->f1, b->h1,
+    RLB_BCUDA(b, rlb::batch::launch_tubes_totals(b->B, b->d_tubes, b->d_par, b->f0, b->f1,
                                                  b->d_tot, b->stream));
     b->launches += 1;
     RLB_BCUDA(b, cudaMemcpyAsync(b->h_tot, b->d_tot, 5 * sizeof(double) * b->B, cudaMemcpyDeviceToHost, b->stream));

@@ -153,8 +153,7 @@ struct Args {
     int nclusters;
     int cluster;            // blocks per cluster
     int np;                 // planes updated per distribution: 19, or 7 under the 1-D symmetry reduction
-    float *f0, *h0, *f1, *h1, *prev;
-    long long ps;
+    float *f0, *f1, *prev;  // population buffers and previous level: blocks of 32 cells (rlb_step_f32.cuh)
 };
 
 // launch the persistent tube kernel (grid = a.nclusters x cluster blocks of
@@ -163,26 +162,23 @@ struct Args {
 // variant's launch bound (256, 384 or 512 threads; threads <= bound).
 cudaError_t launch_tubes(const Args &a, int threads, int bound, int cluster, cudaStream_t s,
                          int *nclusters_out);
-cudaError_t launch_tubes_ca(const Args &a, int threads, int bound, cudaStream_t s, int *nclusters_out);
-cudaError_t launch_tubes_cg(const Args &a, int threads, int bound, int cluster, cudaStream_t s,
-                            int *nclusters_out);
+cudaError_t launch_tubes_19(const Args &a, int threads, int bound, int cluster, cudaStream_t s, int *nclusters_out);
+cudaError_t launch_tubes_7(const Args &a, int threads, int bound, int cluster, cudaStream_t s, int *nclusters_out);
 
 // packed fields <-> tube storage; pack[b] = first packed index of tube b
-cudaError_t launch_tubes_init(int B, int max_nx, const Tube *tubes, const long long *pack, long long ps,
-                              const double *n, const double *T, const double *ux, float *f, float *h,
-                              float *prev, unsigned *status, cudaStream_t s);
+cudaError_t launch_tubes_init(int B, int max_nx, const Tube *tubes, const long long *pack, const double *n,
+                              const double *T, const double *ux, float *f, float *prev, unsigned *status, cudaStream_t s);
 cudaError_t launch_tubes_macro(int B, int max_nx, const Tube *tubes, const long long *pack, const int *par,
-                               long long ps, long long total, const float *f0, const float *h0,
-                               const float *f1, const float *h1, double *out, unsigned *status,
+                               long long total, const float *f0, const float *f1, double *out, unsigned *status,
                                cudaStream_t s);
 // 1-D symmetry reduction: copy every class representative's plane into the
 // planes of the other populations of its class, in each tube's current
 // buffer, so that the full 19-population state is consistent again
-cudaError_t launch_tubes_expand(int B, int max_nx, const Tube *tubes, const int *par, long long ps, float *f0,
-                                float *h0, float *f1, float *h1, cudaStream_t s);
+cudaError_t launch_tubes_expand(int B, int max_nx, const Tube *tubes, const int *par, float *f0, float *f1,
+                                cudaStream_t s);
 // per-tube totals of T^00, T^0x, T^0y, T^0z, N^0: out[5 b + k]
-cudaError_t launch_tubes_totals(int B, const Tube *tubes, const int *par, long long ps, const float *f0,
-                                const float *h0, const float *f1, const float *h1, double *out,
+cudaError_t launch_tubes_totals(int B, const Tube *tubes, const int *par, const float *f0,
+                                const float *f1, double *out,
                                 cudaStream_t s);
 
 }  // namespace batch

@@ -93,40 +93,9 @@ __device__ __forceinline__ int map1(int c, int n, int lo, int hi)
     return c < 0 ? 0 : n - 1;
 }
 
-// one pair of a tube of the batch (planes of stride ps)
-struct Geo {
-    int idx0;            // first cell
-    int x0;
-    bool has1;           // x0 + 1 is inside the tube
-    int oa, oc;          // offsets of the pairs holding x0-2, x0-1 and x0+2, x0+3
-    unsigned xfix;       // XF_*
-};
-
-// Load kinds of the batch.  LD_CA (cached in L1) when only threads of the
-// same block wrote the data (ordered by the block barrier), LD_CG (cached in
-// L2 only) when other blocks of the cluster wrote it on other SMs.
-enum { LD_CA = 1, LD_CG = 2 };
-template <int LD>
-__device__ __forceinline__ f2 ld2(const float *q)
-{
-    const float2 *p = reinterpret_cast<const float2 *>(q);
-    float2 v;
-    if constexpr (LD == LD_CG) v = __ldcg(p);
-    else v = __ldca(p);
-    return f2{v.x, v.y};
-}
-
 // Where the stencil values of one population come from.  get(slot): the pairs
 // at x0-2, x0, x0+2 (slots 0, 1, 2); nb<A, D>(slot): the pair at distance D
 // along axis A, the k-th one that population needs there (slot 3 A + k).
-struct StageSrc {
-    const f2 *s;     // slot 0 of this thread's shared-memory buffer
-    int stride;      // f2 elements between slots
-    __device__ __forceinline__ f2 get(int slot) const { return s[slot * stride]; }
-    template <int A, int D>
-    __device__ __forceinline__ f2 nb(int slot) const { return get(slot); }
-    __device__ __forceinline__ float extra() const { return 0.0f; }
-};
 // values loaded into registers
 struct Sten {
     f2 v[9];
@@ -623,10 +592,10 @@ struct BlockIO {
     }
 };
 
-// Planes of stride ps (the batch's tubes and the bulk-staged grids): the own
-// pair and the previous level
-template <int NP, int LD>
+// Planes of stride ps (the bulk-staged grids): the own pair and the previous
+// level
 struct PlaneIO {
+    static constexpr int NP = 19;
     const StepParams &p;
     const float *f, *h;
     float *fo, *ho, *pv;
@@ -638,12 +607,8 @@ struct PlaneIO {
     __device__ __forceinline__ f2 own() const
     {
         const float *q = (Item<NP, J>::IS_F ? f : h) + Item<NP, J>::I * ps + idx0;
-        if constexpr (LD == 0) {
-            const float2 v = __ldg(reinterpret_cast<const float2 *>(q));
-            return f2{v.x, v.y};
-        } else {
-            return ld2<LD>(q);
-        }
+        const float2 v = __ldg(reinterpret_cast<const float2 *>(q));
+        return f2{v.x, v.y};
     }
     template <int J>
     __device__ __forceinline__ void put(f2 v) const
@@ -664,74 +629,11 @@ struct PlaneIO {
     }
 };
 
-// Asynchronous copies (cp.async, cached in L1) into shared memory, completed
-// per thread by cp.async.wait_group: no other thread reads the slots.
-__device__ __forceinline__ void cp8(unsigned dst, const float *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-constexpr int kStageBufs = 3;                // populations in flight: the one computed and the next ones
-constexpr int kStageAhead = kStageBufs - 1;  // prefetch distance in populations
-
-// Tubes of the batch: the three pairs of each population's stencil are copied
-// into this thread's shared-memory slots kStageAhead populations ahead of
-// their use.  stage = slot 0 of buffer 0 of this thread, sstride = f2
-// elements between slots.
-template <int NP, int LD>
-struct StageIO : PlaneIO<NP, LD> {
-    int oa, oc;
-    f2 *stage;
-    int sstride;
-    unsigned dst0;
-
-    static constexpr int NI = 2 * NP;
-    template <int J>
-    __device__ __forceinline__ void issue() const
-    {
-        using T = Item<NP, J>;
-        constexpr bool xneed = cdir<T::I, 0>() != 0 || (T::IS_F && T::I != 0);
-        const unsigned ss = unsigned(sstride * sizeof(f2));
-        const unsigned d = dst0 + unsigned(J % kStageBufs) * 3 * ss;
-        const float *q = (T::IS_F ? this->f : this->h) + T::I * this->ps + this->idx0;
-        if constexpr (xneed) {
-            cp8(d, q + oa);
-            cp8(d + 2 * ss, q + oc);
-        }
-        cp8(d + ss, q);
-        cp_commit();
-    }
-    __device__ __forceinline__ void begin()
-    {
-        dst0 = unsigned(__cvta_generic_to_shared(stage));
-        for_pops(std::make_integer_sequence<int, kStageAhead>{}, [&](auto jc) { issue<decltype(jc)::value>(); });
-    }
-    template <int S, int J>
-    __device__ __forceinline__ f2 pre()
-    {
-        using T = Item<NP, J>;
-        if constexpr (J + kStageAhead < NI) {
-            issue<J + kStageAhead>();
-            cp_wait<kStageAhead>();
-        } else {
-            cp_wait<NI - 1 - J>();   // the groups issued after item J's
-        }
-        const StageSrc src{stage + (J % kStageBufs) * 3 * sstride, sstride};
-        return streamed2<1, T::IS_F, T::I, 0, false>(src, this->xfix, 0.0f, this->p.f_k1, this->p.f_k2,
-                                                     this->p.f_half_lim, this->kb);
-    }
-};
-
 // 3-D grids staged by bulk copies (rlb_bulk.cuh)
 template <int LAT>
-struct BulkIO : PlaneIO<19, 0> {
+struct BulkIO : PlaneIO {
     Bulk *bk;
-    static constexpr int NP = 19, NI = 38;
+    static constexpr int NI = 38;
     __device__ __forceinline__ void begin() {}
     template <int S, int J>
     __device__ __forceinline__ f2 pre()
@@ -1000,11 +902,12 @@ __device__ __forceinline__ void slab_order(int slab_by, unsigned &bx, unsigned &
 #define RLB_F32_BY 8
 #endif
 
+// threads per block of the 1-D form (us for 200 steps with 32 / 64 / 128: 800
+// cells symmetric 815 / 795 / 736, 8192 cells 1362 / 1398 / 1416)
+constexpr int kTubeThreads = 128;
 constexpr int kParkH = 11;   // f2 slots per thread in shared memory of the parked h coefficients
 // dynamic shared memory of one block of nthr threads
 constexpr size_t park_bytes(int nthr, int dim) { return sizeof(f2) * size_t(nthr) * (kParkH + (dim > 1 ? kEqSlots : 0)); }
-// the batch's blocks add the staged stencils
-constexpr size_t tube_smem_bytes(int nthr) { return sizeof(f2) * size_t(nthr) * (kParkH + 3 * kStageBufs); }
 
 // NP = 14: the 2-D symmetry reduction (DIM = 2, viscous step).  ODDP: nx odd
 // with a periodic x face.  LIN: blocks of one row of 32 BY threads take
@@ -1085,7 +988,7 @@ __global__ void __launch_bounds__(32 * RLB_F32_BY, RLB_F32_MINB)
     // threads per block as the launcher sets them (rlb_step_f32_launch.cuh), a
     // compile-time constant so that the shared-memory slots of this thread
     // sit at fixed offsets from one base address
-    constexpr int nthr = (DIM == 1 && !LIN) ? 128 : 32 * RLB_F32_BY;
+    constexpr int nthr = (DIM == 1 && !LIN) ? kTubeThreads : 32 * RLB_F32_BY;
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     update_pair<EULER, (DIM > 1), NP, LAT, REC64>(p, io, has1, p.f_eta_over_s, s_park + tid, nthr);
 }

@@ -39,8 +39,8 @@ cudaError_t launch_f32(const StepParams &p, const float *f, float *fo, float *pr
         block = dim3(32 * RLB_F32_BY, 1, 1);
         grid = dim3(unsigned((pairs + 32 * RLB_F32_BY - 1) / (32 * RLB_F32_BY)), 1, 1);
     } else if (DIM == 1) {
-        block = dim3(128, 1, 1);
-        grid = dim3((npairs + 127) / 128, 1, 1);
+        block = dim3(f32::kTubeThreads, 1, 1);
+        grid = dim3((npairs + f32::kTubeThreads - 1) / f32::kTubeThreads, 1, 1);
     } else {
         // 32 x 8 threads (64 x 8 cells), two blocks per SM at <= 128 registers:
         // the best of a sweep over block shapes and register caps on GB300
