@@ -122,7 +122,7 @@ typedef struct {
                               * on grids that allow it (3-D, viscous, extended lattice, nx a
                               * multiple of 64, ny of 8, x faces not periodic) the block stages
                               * each population's stencil tile into shared memory by tensor-map
-                              * bulk copies instead of each thread staging its own, when the
+                              * bulk copies instead of each thread loading its own, when the
                               * driver provides the tensor-map encoder (see rlb_step_kernel).
                               * The results are the same bit for bit. */
     int symmetry_2d;         /* 1 (grids with nz = 1 < ny, either precision, viscous step): exact 2-D
@@ -194,8 +194,9 @@ RLB_API rlb_status rlb_check_config(const rlb_grid *grid, int Q, double eta_over
  * this small alpha: at zeta/s <= 0.1, alpha <= 1.2e-3, far below the
  * alpha = 0.15 .. 0.2 the paper's runs use for stability.  To set the term
  * that keeps fast flows physical, give alpha_override. 
- * opts may be NULL (defaults).  Allocates 2 x 38 population planes, 5
- * previous-level planes and scratch on the device; *out receives the handle
+ * opts may be NULL (defaults).  Allocates 2 x 38 populations, 5
+ * previous-level values (FP32 storage: rows padded to an even number of cells)
+ * and scratch on the device; *out receives the handle
  * (NULL on failure).  Errors: RLB_E_INVALID, RLB_E_UNSTABLE, RLB_E_NOMEM,
  * RLB_E_CUDA. */
 RLB_API rlb_status rlb_create(const rlb_grid *grid, int Q, double eta_over_s, double zeta_over_s,
@@ -287,10 +288,10 @@ RLB_API const char *rlb_status_string(int status);
  * copies: thread_mapping 3, viscous step, extended lattice, nx a multiple
  * of 64, ny of 8, x faces not periodic, tensor maps made at rlb_create),
  * "fp32_tiles" (tiles of
- * 64 x 8 cells, each thread loading its own stencil, staged by asynchronous
- * copies in the viscous step), "fp32_linear", "fp32_1d", "fp32_rec64" (recovery_fp64),
- * "fp64_tiles", "fp64_linear", "fp64_small" (blocks of one to four warps
- * on grids with fewer cells than one block per SM), "fp64_1d".  The
+ * 64 x 8 cells, each thread loading its own stencil into registers), "fp32_linear", "fp32_1d", "fp32_rec64" (recovery_fp64),
+ * "fp64_tiles", "fp64_linear", "fp64_small" (grids with fewer cells than
+ * one block of 128 per SM: four warps share 32 cells; in Euler mode blocks of
+ * one to four warps), "fp64_1d".  The
  * results are the same whichever kernel runs.  NULL ctx: "none". */
 RLB_API const char *rlb_step_kernel(const rlb_ctx *ctx);
 
@@ -393,7 +394,10 @@ RLB_API rlb_status rlb_batch_init(rlb_batch *b, const double *n, const double *T
 /* Advance tube b by nsteps[b] steps of Eq. 57 (host array of B counts in
  * [0, 2^31 - 1]; 0 leaves a tube unchanged) in one launch of the persistent
  * kernel, replayed from a CUDA graph.  The job plan is rebuilt when the step
- * counts or the tuning change.  Waits for the launch and returns
+ * counts or the tuning change.  Unless rlb_batch_set_tuning or
+ * rlb_batch_autotune set a launch shape, the first call chooses one for its
+ * step counts from the plans of several shapes and measured pass times, and
+ * later calls keep it.  Waits for the launch and returns
  * RLB_E_NONPHYSICAL if any cell of any step was non-physical. */
 RLB_API rlb_status rlb_batch_step(rlb_batch *b, const long long *nsteps);
 

@@ -76,7 +76,7 @@ cudaError_t launch_step_f32(const StepParams &p, int dim, int euler, const float
 // (blocked storage: h and ho are not used; with maps: planes)
 // the FP32-storage step on eligible 3-D grids with its stencil tiles staged by
 // bulk copies (rlb_step_f32_bulk.cu); it needs the tensor maps of the buffers
-// it reads (launch_step_f32 runs the per-thread staged kernel without them)
+// it reads (launch_step_f32 runs the per-thread kernel without them)
 bool f32_bulk_eligible(const StepParams &p, int dim, int euler);
 // encode the maps of the planes at f and h (cudaSuccess, or the failure)
 cudaError_t make_tile_maps(const StepParams &p, const float *f, const float *h, TileMaps *out);

@@ -239,7 +239,7 @@ __device__ __forceinline__ void flag(const StepParams &p, unsigned bits)
 // NP = 7 or 14: the 1-D or 2-D symmetry reduction (rlb_classes.cuh); only
 // the class representatives' planes are read and written
 //
-// Bound by the FP64 pipe (621 operations a cell, 1208 before the fixed-point
+// Bound by the FP64 pipe (631 operations a cell, 1208 before the fixed-point
 // streaming and the shared sums) together with the latency of its chains, so
 // warps count: at 128 registers (four blocks of 128 per SM; the own
 // populations are loaded again rather than held) the 256 x 128 x 128 cloud

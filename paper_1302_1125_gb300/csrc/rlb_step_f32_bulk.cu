@@ -4,7 +4,7 @@
 // planes, extended lattice, nx a multiple of 64 and ny a multiple of 8 (every
 // block a full 64 x 8 tile, so that all its threads take part in the
 // barriers), x faces not periodic, and rlb_options.thread_mapping = 3 (an
-// option); the launcher in rlb_step_f32.cu runs the per-thread staged kernel
+// option); the launcher in rlb_step_f32.cu runs the per-thread kernel
 // otherwise, and also when the tensor maps could not be made.
 #include <cudaTypedefs.h>   // PFN_cuTensorMapEncodeTiled
 
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kBulkThreads, 2)
     b.warp = ty;
     b.lane = tx;
     unsigned bx = blockIdx.x, by = blockIdx.y, bz = blockIdx.z;
-    slab_order(p.slab_by, bx, by, bz);   // the per-thread staged kernel's block order
+    slab_order(p.slab_by, bx, by, bz);   // the per-thread kernel's block order
     b.x0t = 64 * int(bx);
     b.y0 = 8 * int(by);
     b.z = int(bz);
