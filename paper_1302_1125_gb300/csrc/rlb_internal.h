@@ -33,7 +33,8 @@ struct StepParams {
 };
 
 // launch a kernel that calls grid_wait (rlb_device.cuh) so that it may start
-// while the kernel before it on the stream still runs
+// while the kernel before it on the stream still runs; a refused launch is
+// reported here and not again by the caller's next check of the last error
 template <typename... P, typename... A>
 cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
 {
@@ -47,7 +48,9 @@ cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 // Storage of a grid's populations: planes of stride ps (FP64 form; FP32 grids
