@@ -41,59 +41,54 @@ __device__ __forceinline__ T nbr(const T *q, int idx, const AxisNbr &a, int k, T
     return ((a.ghost >> k) & 1u) ? ghost : ldg(q + idx + a.off[k]);
 }
 
-// Streaming terms of one population along axis A (Eqs. 47-53): the
-// accumulator acc receives minus dt (c0/ct) times the conservative minmod
-// flux difference h^a(x) - h^a(x - e_a); for f with i != 0 the neighbour sum
-// s receives q(x + e_A) + q(x - e_A) of the bulk term's second difference
-// (assigned on the first axis, FIRST).
-template <typename T, bool IS_F, int I, int A, int LAT, bool FIRST>
-__device__ __forceinline__ void axis_terms(const T *q, int idx, const AxisNbr &an, T qc, T ghost,
-                                           T k1, T k2, T hl, T &acc, T &s)
+// f + streaming (+ bulk) of a population: the explicit part of Eq. 57.  v[a]:
+// its values at -1, +1 and, upwind, -2 or +2 along axis a; way: the
+// population's steps along the axes and whether it carries the bulk term
+// (way_of).  Along each axis it moves on, the sum receives minus dt (c0/ct)
+// times the conservative minmod flux difference h^a(x) - h^a(x - e_a) (Eqs.
+// 47-53).  The bulk term's central second difference sum_A [q(x + e_A) -
+// 2 q(x) + q(x - e_A)] is taken as s - 2 DIM q(x) in one fused operation
+// (exact coefficients, so that its sum over a periodic grid carries no
+// systematic rounding).
+constexpr int kWayBulk = 512;
+constexpr int way_of(int cx, int cy, int cz, bool bulk)
 {
-    constexpr int c = cdir<I, A, LAT>();
-    constexpr bool need_lap = IS_F && I != 0;
-    auto add_s = [&](T qm1, T qp1) {
-        if constexpr (need_lap) {
-            if constexpr (FIRST) s = qp1 + qm1;
-            else s += qp1 + qm1;
-        }
-    };
-    if constexpr (c > 0) {
-        const T qm2 = nbr(q, idx, an, 0, ghost);
-        const T qm1 = nbr(q, idx, an, 1, ghost);
-        const T qp1 = nbr(q, idx, an, 2, ghost);
-        const T d0 = qm1 - qm2, d1 = qc - qm1, d2 = qp1 - qc;
-        const T D = fma(hl, minmod(d2, d1) - minmod(d1, d0), d1);
-        acc = fma(-(c == 1 ? k1 : k2), D, acc);
-        add_s(qm1, qp1);
-    } else if constexpr (c < 0) {
-        const T qm1 = nbr(q, idx, an, 1, ghost);
-        const T qp1 = nbr(q, idx, an, 2, ghost);
-        const T qp2 = nbr(q, idx, an, 3, ghost);
-        const T e0 = qc - qm1, e1 = qp1 - qc, e2 = qp2 - qp1;
-        const T D = fma(-hl, minmod(e1, e2) - minmod(e0, e1), e1);
-        acc = fma(c == -1 ? k1 : k2, D, acc);
-        add_s(qm1, qp1);
-    } else if constexpr (need_lap) {
-        add_s(nbr(q, idx, an, 1, ghost), nbr(q, idx, an, 2, ghost));
-    }
+    return (cx + 2) | (cy + 2) << 3 | (cz + 2) << 6 | (bulk ? kWayBulk : 0);
 }
-
-// f + streaming (+ bulk) for population I: the explicit part of Eq. 57.  The
-// bulk term's central second difference sum_A [q(x + e_A) - 2 q(x) + q(x - e_A)]
-// is taken as s - 2 DIM q(x) in one fused operation (exact coefficients, so
-// that its sum over a periodic grid carries no systematic rounding).
-template <typename T, int DIM, bool IS_F, int I, int LAT>
-__device__ __forceinline__ T streamed(const T *q, int idx, const AxisNbr (&am)[3], T qc, T ghost,
-                                      T k1, T k2, T hl, T kbulk)
+struct Sten64 {
+    double v[3][3];
+};
+template <int DIM>
+__device__ __forceinline__ double streamed(const Sten64 &q, double qc, double k1, double k2, double hl, double kbulk,
+                                           int way)
 {
-    constexpr bool need_lap = IS_F && I != 0;
-    T acc = qc, s = T(0);
-    axis_terms<T, IS_F, I, 0, LAT, true>(q, idx, am[0], qc, ghost, k1, k2, hl, acc, s);
-    if constexpr (DIM > 1) axis_terms<T, IS_F, I, 1, LAT, false>(q, idx, am[1], qc, ghost, k1, k2, hl, acc, s);
-    if constexpr (DIM > 2) axis_terms<T, IS_F, I, 2, LAT, false>(q, idx, am[2], qc, ghost, k1, k2, hl, acc, s);
-    if constexpr (need_lap) acc = fma(kbulk, fma(T(-2 * DIM), qc, s), acc);
+    double acc = qc, s = 0.0;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        const int c = ((way >> 3 * a) & 7) - 2;
+        const double (&v)[3] = q.v[a];
+        if (c > 0) {
+            const double d0 = v[0] - v[2], d1 = qc - v[0], d2 = v[1] - qc;
+            const double D = fma(hl, minmod(d2, d1) - minmod(d1, d0), d1);
+            acc = fma(-(c == 1 ? k1 : k2), D, acc);
+        } else if (c < 0) {
+            const double e0 = qc - v[0], e1 = v[1] - qc, e2 = v[2] - v[1];
+            const double D = fma(-hl, minmod(e1, e2) - minmod(e0, e1), e1);
+            acc = fma(c == -1 ? k1 : k2, D, acc);
+        }
+        if (way & kWayBulk) {
+            if (a == 0) s = v[1] + v[0];
+            else s += v[1] + v[0];
+        }
+    }
+    if (way & kWayBulk) acc = fma(kbulk, fma(double(-2 * DIM), qc, s), acc);
     return acc;
+}
+template <int DIM>
+__device__ __noinline__ double streamed_called(const Sten64 q, double qc, double k1, double k2, double hl, double kbulk,
+                                               int way)
+{
+    return streamed<DIM>(q, qc, k1, k2, hl, kbulk, way);
 }
 
 // ---------------------------------------------------------------------------
@@ -111,8 +106,16 @@ __device__ __forceinline__ T streamed(const T *q, int idx, const AxisNbr (&am)[3
 // are exact (in FP64 each rounds).  Headroom: values < 2^59, differences <
 // 2^60, 2 D per axis < 2^62, two axes and the Laplacian (< 6 2^60) < 2^63.
 // Stencils with a wider spread of exponents, zeros, subnormal or non-finite
-// values take the FP64 form above.
+// values take the FP64 form above: inlined at every population (FX_INLINE), or
+// one function that they all call (FX_CALL).  Inlined it makes the code of a
+// step about twice as long, and a kernel with a warp or two per scheduler waits
+// for instructions: the four-warp kernel (step_split_kernel) takes 22 us a step
+// on 64 x 64 cells inlined, 18.2 called, and in 3-D 151 registers, with which a
+// fourth block does not fit on an SM (32 x 32 x 18 cells 64 us), or 126 (34 us).
+// With four warps per scheduler the call costs more than it saves (1024 x 512
+// cells 690 us inlined, 756 called).
 // ---------------------------------------------------------------------------
+enum { FX_INLINE, FX_CALL };
 constexpr int kFxGap = 6;
 
 __device__ __forceinline__ long long to_fx(double x, int e0)   // e0 = E - kFxGap
@@ -139,7 +142,7 @@ __device__ __forceinline__ double fx_scaled(double k, int e)
 
 // gap: kFxGap, or -1 when a prefactor is too small for fx_scaled (the FP64 form
 // is taken); lim: -1 for the minmod limiter, 0 for none
-template <int DIM, bool IS_F, int I, int LAT>
+template <int DIM, bool IS_F, int I, int LAT, int FORM>
 __device__ __forceinline__ double streamed_fx(const double *q, int idx, const AxisNbr (&am)[3], double qc, double ghost,
                                               double k1, double k2, double hl, double kbulk, int gap, long long lim)
 {
@@ -149,27 +152,36 @@ __device__ __forceinline__ double streamed_fx(const double *q, int idx, const Ax
     if constexpr (!moves && !need_lap) {
         return qc;
     } else {
-        // v[a]: the values at -1, +1 and, upwind, -2 or +2 along axis a
-        double v[3][3];
+        Sten64 st = {};
+        double (&v)[3][3] = st.v;
+        auto load = [&](auto &&take) {
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                if (c[a] != 0 || need_lap) {
+                    v[a][0] = take(nbr(q, idx, am[a], 1, ghost));
+                    v[a][1] = take(nbr(q, idx, am[a], 2, ghost));
+                }
+                if (c[a] > 0) v[a][2] = take(nbr(q, idx, am[a], 0, ghost));
+                if (c[a] < 0) v[a][2] = take(nbr(q, idx, am[a], 3, ghost));
+            }
+        };
+        constexpr int way = way_of(c[0], c[1], c[2], need_lap);
         unsigned hx = unsigned(__double2hiint(qc)) & 0x7fffffffu, hn = hx;
-        auto take = [&](double x) {
+        load([&](double x) {
             const unsigned h = unsigned(__double2hiint(x)) & 0x7fffffffu;
             hx = max(hx, h);
             hn = min(hn, h);
             return x;
-        };
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            if (c[a] != 0 || need_lap) {
-                v[a][0] = take(nbr(q, idx, am[a], 1, ghost));
-                v[a][1] = take(nbr(q, idx, am[a], 2, ghost));
-            }
-            if (c[a] > 0) v[a][2] = take(nbr(q, idx, am[a], 0, ghost));
-            if (c[a] < 0) v[a][2] = take(nbr(q, idx, am[a], 3, ghost));
-        }
+        });
         const int E = int(hx >> 20), En = int(hn >> 20);
-        if (E - En > gap || E >= 0x7ff || En < 512)
-            return streamed<double, DIM, IS_F, I, LAT>(q, idx, am, qc, ghost, k1, k2, hl, kbulk);
+        if (E - En > gap || E >= 0x7ff || En < 512) {
+            if constexpr (FORM == FX_CALL) {
+                return streamed_called<DIM>(st, qc, k1, k2, hl, kbulk, way);
+            } else {
+                load([](double x) { return x; });   // again, rather than held for a branch that is seldom taken
+                return streamed<DIM>(st, qc, k1, k2, hl, kbulk, way);
+            }
+        }
         const int e0 = E - kFxGap;
         const long long fc = to_fx(qc, e0);
         long long T = 0, L = 0;
@@ -344,8 +356,8 @@ __global__ void __launch_bounds__(128, RLB_F64_MINB) step_kernel(const StepParam
             for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 constexpr int I = rep<NP>(k);
-                const T pre = streamed_fx<DIM, true, I, LAT>(f + I * ps, idx, am, ldg(f + I * ps + idx), T(p.ghost_f[I]), k1, k2, hl,
-                                                             kbulk, gap, lim);
+                const T pre = streamed_fx<DIM, true, I, LAT, FX_INLINE>(f + I * ps, idx, am, ldg(f + I * ps + idx),
+                                                                        T(p.ghost_f[I]), k1, k2, hl, kbulk, gap, lim);
                 fo[I * ps + idx] = fma(kap, eq_pop<I>(kf) - pre, pre);
             });
         }
@@ -362,8 +374,8 @@ __global__ void __launch_bounds__(128, RLB_F64_MINB) step_kernel(const StepParam
             for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 constexpr int I = rep<NP>(k);
-                const T pre = streamed_fx<DIM, false, I, LAT>(h + I * ps, idx, am, ldg(h + I * ps + idx), T(p.ghost_h[I]), k1, k2, hl,
-                                                              kbulk, gap, lim);
+                const T pre = streamed_fx<DIM, false, I, LAT, FX_INLINE>(h + I * ps, idx, am, ldg(h + I * ps + idx),
+                                                                         T(p.ghost_h[I]), k1, k2, hl, kbulk, gap, lim);
                 ho[I * ps + idx] = fma(kap, eq_pop<I>(kh) - pre, pre);
             });
         }
@@ -373,14 +385,14 @@ __global__ void __launch_bounds__(128, RLB_F64_MINB) step_kernel(const StepParam
         for_pops(RLB_POPS, [&](auto ic) {
             constexpr int I = decltype(ic)::value;
             const T qc = ldg(f + I * ps + idx);
-            const double fv = double(streamed_fx<DIM, true, I, LAT>(f + I * ps, idx, am, qc, T(p.ghost_f[I]), k1, k2,
+            const double fv = double(streamed_fx<DIM, true, I, LAT, FX_INLINE>(f + I * ps, idx, am, qc, T(p.ghost_f[I]), k1, k2,
                                                                     hl, kbulk, gap, lim));
             sf += fv;
             if constexpr (cdir<I, 0, LAT>() != 0) mx += double(cdir<I, 0, LAT>()) * fv;
             if constexpr (cdir<I, 1, LAT>() != 0) my += double(cdir<I, 1, LAT>()) * fv;
             if constexpr (cdir<I, 2, LAT>() != 0) mz += double(cdir<I, 2, LAT>()) * fv;
             const T qh = ldg(h + I * ps + idx);
-            sh += double(streamed_fx<DIM, false, I, LAT>(h + I * ps, idx, am, qh, T(p.ghost_h[I]), k1, k2, hl, kbulk,
+            sh += double(streamed_fx<DIM, false, I, LAT, FX_INLINE>(h + I * ps, idx, am, qh, T(p.ghost_h[I]), k1, k2, hl, kbulk,
                                                          gap, lim));
         });
         Macro mt;
@@ -409,7 +421,7 @@ __global__ void __launch_bounds__(128, RLB_F64_MINB) step_kernel(const StepParam
 // scheduler's share of the pipe, one per 64 clocks, so on a grid with fewer
 // warps of cells than schedulers a step takes the time of one warp's FP64
 // instructions whatever the number of SMs (31 us a step on an 800-cell tube;
-// 15 us here).
+// 13 us here).
 // Here the four warps of a block, one per scheduler, share 32 cells: each
 // takes the f and h of one part (part_of), and between the moments and the
 // relaxation warp 3 recovers the macroscopic state while the others form the
@@ -542,7 +554,7 @@ __global__ void __launch_bounds__(128) step_split_kernel(const StepParams p, con
     auto explicit_parts = [&]() {
         items([&](auto Jc, auto jc) {
             constexpr int J = decltype(Jc)::value, j = decltype(jc)::value, I = rep<NP>(J < NP ? J : J - NP);
-            pre[j] = streamed_fx<DIM, (J < NP), I, LAT>((J < NP ? f : h) + I * ps, idx, am, own[j],
+            pre[j] = streamed_fx<DIM, (J < NP), I, LAT, FX_CALL>((J < NP ? f : h) + I * ps, idx, am, own[j],
                                                         J < NP ? p.ghost_f[I] : p.ghost_h[I], k1, k2, hl, kbulk, gap, lim);
         });
     };

@@ -20,20 +20,34 @@ inline int sm_count()
     return n;
 }
 
+// Grids that the small-grid kernels take, unless the mapping asks for tiles (1;
+// 3: FP32 tiles): fewer than 128 cells per SM, four blocks of 32 cells.  us a
+// step on 152 SMs: 1-D 16.3 at 64 cells an SM, 25.8 at 96, 26.0 at 128 (tiles of
+// 128 cells 33), 2-D 20.6, 30.2, 30.0 (45.6), 3-D 32.2 at 42, 33.8 at 96, 34.0 at
+// 121 (56).  Under the 1-D reduction 80 cells per SM: five of its blocks fit on
+// an SM, and up to two and a half to an SM those of the next step (which start
+// while a step runs) all find room.  Beyond, the SMs that finish first take the
+// rest, up to five to an SM: 15.0 at 79 cells per SM, 22.5 from 86 on (tiles 18.0).
+inline bool f64_small(const StepParams &p)
+{
+    const long long cells = (long long)p.nx * p.ny * p.nz, nsm = sm_count();
+    return (p.sym == 1 ? cells <= 80 * nsm : cells < 128 * nsm) && p.mapping != 1 && p.mapping != 3;
+}
+
 template <typename T, int DIM, bool EULER, int LAT, int NP>
 cudaError_t launch_step_np(const StepParams &p, const T *f, const T *h, T *fo, T *ho, T *prev,
                           cudaStream_t s)
 {
     const long long cells = (long long)p.nx * p.ny * p.nz;
-    // Grids with fewer cells than one block of 128 per SM: four warps to 32
-    // cells (step_split_kernel); in Euler mode blocks of one to four warps of
-    // consecutive cells (x-fastest order) spread the cells over more SMs.
-    const int nsm = sm_count();
-    if (cells < 128LL * nsm && p.mapping != 1 && p.mapping != 3) {   // 3: tiles (FP32: bulk-staged)
+    // Small grids: four warps to 32 cells (step_split_kernel); in Euler mode
+    // blocks of one to four warps of consecutive cells (x-fastest order) spread
+    // the cells over more SMs.
+    if (f64_small(p)) {
         if constexpr (!EULER) {
             return launch_overlapped(step_split_kernel<DIM, LAT, NP>, unsigned((cells + 31) / 32), dim3(32, 4, 1), 0, s, p,
                                      f, h, fo, ho, prev);
         } else {
+            const int nsm = sm_count();
             int bs = int(((cells + nsm - 1) / nsm + 31) / 32 * 32);
             bs = bs < 32 ? 32 : (bs > 128 ? 128 : bs);
             const unsigned nb = unsigned((cells + bs - 1) / bs);
