@@ -113,9 +113,13 @@ __device__ __noinline__ double streamed_called(const Sten64 q, double qc, double
 // on 64 x 64 cells inlined, 18.2 called, and in 3-D 151 registers, with which a
 // fourth block does not fit on an SM (32 x 32 x 18 cells 64 us), or 126 (34 us).
 // With four warps per scheduler the call costs more than it saves (1024 x 512
-// cells 690 us inlined, 756 called).
+// cells 690 us inlined, 756 called), but not in Euler mode, whose streaming is
+// all in one loop (64 x 64 cells 34.7 and 27.4, 256 x 128 x 128 5080 and 4310).
+// FX_NONE: the FP64 form alone, for 1-D tubes in Euler mode with one warp per
+// scheduler, which gain nothing from the fixed point (800 cells 23.5 us called,
+// 20.7 so).
 // ---------------------------------------------------------------------------
-enum { FX_INLINE, FX_CALL };
+enum { FX_INLINE, FX_CALL, FX_NONE };
 constexpr int kFxGap = 6;
 
 __device__ __forceinline__ long long to_fx(double x, int e0)   // e0 = E - kFxGap
@@ -166,6 +170,11 @@ __device__ __forceinline__ double streamed_fx(const double *q, int idx, const Ax
             }
         };
         constexpr int way = way_of(c[0], c[1], c[2], need_lap);
+        auto same = [](double x) { return x; };
+        if constexpr (FORM == FX_NONE) {
+            load(same);
+            return streamed<DIM>(st, qc, k1, k2, hl, kbulk, way);
+        }
         unsigned hx = unsigned(__double2hiint(qc)) & 0x7fffffffu, hn = hx;
         load([&](double x) {
             const unsigned h = unsigned(__double2hiint(x)) & 0x7fffffffu;
@@ -178,7 +187,7 @@ __device__ __forceinline__ double streamed_fx(const double *q, int idx, const Ax
             if constexpr (FORM == FX_CALL) {
                 return streamed_called<DIM>(st, qc, k1, k2, hl, kbulk, way);
             } else {
-                load([](double x) { return x; });   // again, rather than held for a branch that is seldom taken
+                load(same);   // again, rather than held for a branch that is seldom taken
                 return streamed<DIM>(st, qc, k1, k2, hl, kbulk, way);
             }
         }
@@ -260,7 +269,7 @@ __device__ __forceinline__ void flag(const StepParams &p, unsigned bits)
 #ifndef RLB_F64_MINB
 #define RLB_F64_MINB 4
 #endif
-template <typename T, int DIM, bool EULER, int LAT, bool LIN = false, int NP = 19>
+template <typename T, int DIM, bool EULER, int LAT, bool LIN = false, int NP = 19, int FORM = EULER ? FX_CALL : FX_INLINE>
 __global__ void __launch_bounds__(128, RLB_F64_MINB) step_kernel(const StepParams p, const T *__restrict__ f,
                                                    const T *__restrict__ h, T *__restrict__ fo,
                                                    T *__restrict__ ho, T *__restrict__ prev)
@@ -356,8 +365,8 @@ __global__ void __launch_bounds__(128, RLB_F64_MINB) step_kernel(const StepParam
             for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 constexpr int I = rep<NP>(k);
-                const T pre = streamed_fx<DIM, true, I, LAT, FX_INLINE>(f + I * ps, idx, am, ldg(f + I * ps + idx),
-                                                                        T(p.ghost_f[I]), k1, k2, hl, kbulk, gap, lim);
+                const T pre = streamed_fx<DIM, true, I, LAT, FORM>(f + I * ps, idx, am, ldg(f + I * ps + idx),
+                                                                   T(p.ghost_f[I]), k1, k2, hl, kbulk, gap, lim);
                 fo[I * ps + idx] = fma(kap, eq_pop<I>(kf) - pre, pre);
             });
         }
@@ -374,8 +383,8 @@ __global__ void __launch_bounds__(128, RLB_F64_MINB) step_kernel(const StepParam
             for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 constexpr int I = rep<NP>(k);
-                const T pre = streamed_fx<DIM, false, I, LAT, FX_INLINE>(h + I * ps, idx, am, ldg(h + I * ps + idx),
-                                                                         T(p.ghost_h[I]), k1, k2, hl, kbulk, gap, lim);
+                const T pre = streamed_fx<DIM, false, I, LAT, FORM>(h + I * ps, idx, am, ldg(h + I * ps + idx),
+                                                                    T(p.ghost_h[I]), k1, k2, hl, kbulk, gap, lim);
                 ho[I * ps + idx] = fma(kap, eq_pop<I>(kh) - pre, pre);
             });
         }
@@ -385,15 +394,15 @@ __global__ void __launch_bounds__(128, RLB_F64_MINB) step_kernel(const StepParam
         for_pops(RLB_POPS, [&](auto ic) {
             constexpr int I = decltype(ic)::value;
             const T qc = ldg(f + I * ps + idx);
-            const double fv = double(streamed_fx<DIM, true, I, LAT, FX_INLINE>(f + I * ps, idx, am, qc, T(p.ghost_f[I]), k1, k2,
-                                                                    hl, kbulk, gap, lim));
+            const double fv = streamed_fx<DIM, true, I, LAT, FORM>(f + I * ps, idx, am, qc, T(p.ghost_f[I]), k1, k2, hl,
+                                                                   kbulk, gap, lim);
             sf += fv;
             if constexpr (cdir<I, 0, LAT>() != 0) mx += double(cdir<I, 0, LAT>()) * fv;
             if constexpr (cdir<I, 1, LAT>() != 0) my += double(cdir<I, 1, LAT>()) * fv;
             if constexpr (cdir<I, 2, LAT>() != 0) mz += double(cdir<I, 2, LAT>()) * fv;
             const T qh = ldg(h + I * ps + idx);
-            sh += double(streamed_fx<DIM, false, I, LAT, FX_INLINE>(h + I * ps, idx, am, qh, T(p.ghost_h[I]), k1, k2, hl, kbulk,
-                                                         gap, lim));
+            sh += streamed_fx<DIM, false, I, LAT, FORM>(h + I * ps, idx, am, qh, T(p.ghost_h[I]), k1, k2, hl, kbulk, gap,
+                                                        lim);
         });
         Macro mt;
         const bool ok = recover(Lat<LAT>::xi0sq * sf, Lat<LAT>::xi0 * mx, Lat<LAT>::xi0 * my, Lat<LAT>::xi0 * mz, Lat<LAT>::xi0 * sh, mt);

@@ -28,11 +28,11 @@ inline int sm_count()
 // an SM, and up to two and a half to an SM those of the next step (which start
 // while a step runs) all find room.  Beyond, the SMs that finish first take the
 // rest, up to five to an SM: 15.0 at 79 cells per SM, 22.5 from 86 on (tiles 18.0).
-inline bool f64_small(const StepParams &p)
+inline bool f64_below(const StepParams &p, int cells_per_sm)
 {
-    const long long cells = (long long)p.nx * p.ny * p.nz, nsm = sm_count();
-    return (p.sym == 1 ? cells <= 80 * nsm : cells < 128 * nsm) && p.mapping != 1 && p.mapping != 3;
+    return (long long)p.nx * p.ny * p.nz < (long long)cells_per_sm * sm_count();
 }
+inline bool f64_small(const StepParams &p) { return f64_below(p, p.sym == 1 ? 80 : 128) && p.mapping != 1 && p.mapping != 3; }
 
 template <typename T, int DIM, bool EULER, int LAT, int NP>
 cudaError_t launch_step_np(const StepParams &p, const T *f, const T *h, T *fo, T *ho, T *prev,
@@ -42,30 +42,33 @@ cudaError_t launch_step_np(const StepParams &p, const T *f, const T *h, T *fo, T
     // Small grids: four warps to 32 cells (step_split_kernel); in Euler mode
     // blocks of one to four warps of consecutive cells (x-fastest order) spread
     // the cells over more SMs.
-    if (f64_small(p)) {
-        if constexpr (!EULER) {
+    int bs = 128;
+    const bool small = f64_small(p);
+    if constexpr (!EULER) {
+        if (small)
             return launch_overlapped(step_split_kernel<DIM, LAT, NP>, unsigned((cells + 31) / 32), dim3(32, 4, 1), 0, s, p,
                                      f, h, fo, ho, prev);
-        } else {
-            const int nsm = sm_count();
-            int bs = int(((cells + nsm - 1) / nsm + 31) / 32 * 32);
-            bs = bs < 32 ? 32 : (bs > 128 ? 128 : bs);
-            const unsigned nb = unsigned((cells + bs - 1) / bs);
-            if constexpr (DIM == 1) return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP>, nb, bs, 0, s, p, f, h, fo, ho, prev);
-            else return launch_overlapped(step_kernel<T, DIM, EULER, LAT, true, NP>, nb, bs, 0, s, p, f, h, fo, ho, prev);
-        }
+    } else if (small) {
+        const int nsm = sm_count();
+        bs = int(((cells + nsm - 1) / nsm + 31) / 32 * 32);
+        bs = bs < 32 ? 32 : (bs > 128 ? 128 : bs);
     }
+    const unsigned nb = unsigned((cells + bs - 1) / bs);
     if constexpr (DIM == 1) {
-        return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP>, (p.nx + 127) / 128, 128, 0, s, p, f, h, fo, ho,
-                                 prev);
+        if constexpr (EULER) {
+            // (whatever the mapping, so that its kernels agree bit for bit)
+            if (f64_below(p, 128))
+                return launch_overlapped(step_kernel<T, 1, true, LAT, false, NP, FX_NONE>, nb, bs, 0, s, p, f, h, fo, ho,
+                                         prev);
+        }
+        return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP>, nb, bs, 0, s, p, f, h, fo, ho, prev);
     } else {
         // tiles of 32 x 4 cells when nx and ny fill them, else 128 consecutive
         // cells of the x-fastest order per block
         const long long tiles_x = (p.nx + 31) / 32, tiles_y = (p.ny + 3) / 4;
         const double fill = double(p.nx) * p.ny / double(tiles_x * 32 * tiles_y * 4);
-        if (p.mapping == 2 || (p.mapping == 0 && fill < 0.97)) {
-            return launch_overlapped(step_kernel<T, DIM, EULER, LAT, true, NP>, unsigned((cells + 127) / 128), 128, 0, s,
-                                     p, f, h, fo, ho, prev);
+        if (small || p.mapping == 2 || (p.mapping == 0 && fill < 0.97)) {
+            return launch_overlapped(step_kernel<T, DIM, EULER, LAT, true, NP>, nb, bs, 0, s, p, f, h, fo, ho, prev);
         } else {
             const dim3 grid(unsigned(tiles_x), unsigned(tiles_y), p.nz);
             return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP>, grid, dim3(32, 4, 1), 0, s, p, f, h, fo,

@@ -54,3 +54,15 @@ def test_the_automatic_kernel_is_not_the_slower_one(dims, kw):
     for a, b in zip(auto.get_state(), tiles.get_state()):
         assert np.array_equal(a, b)
     assert us_a_step(auto) <= 1.05 * us_a_step(tiles)
+
+
+# rows of one pair, ragged blocks, the last size below the bound and one above it
+@pytest.mark.parametrize("dims", [(2, 1, 1), (33, 1, 1), (19455, 1, 1), (20000, 1, 1), (33, 17, 1), (17, 9, 7),
+                                  (32, 32, 19)])
+@pytest.mark.parametrize("model", [0, 1])
+def test_euler_mappings_agree_bit_for_bit(dims, model):
+    states = [grid(dims, m, model=model, euler_mode=1).step(5).get_state()
+              for m in (rlb.MAPPING_AUTO, rlb.MAPPING_TILES, rlb.MAPPING_LINEAR)]
+    for other in states[1:]:
+        for a, b in zip(states[0], other):
+            assert np.array_equal(a, b)
