@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(MAXT, 1) tubes_kernel(const Args a)
                     // the slots of the shared-memory array are MAXT apart (the
                     // launch bound, a compile-time constant: fixed offsets
                     // from one base address), whatever blockDim.x <= MAXT is
-                    f32::update_pair<false, false, NP, 0, false>(a.p, io, x0 + 1 < nx, s_eos[i], s_dyn + threadIdx.x, MAXT);
+                    f32::update_pair<false, f32::EQ_FOLD, NP, 0, false>(a.p, io, x0 + 1 < nx, s_eos[i], s_dyn + threadIdx.x, MAXT);
                 }
             }
             if (C > 1) cluster_barrier();

@@ -295,6 +295,20 @@ __device__ __forceinline__ void park_eq(const W2 &e, f2 *q, int stride)
     q[8 * stride] = e.d0 + (e.dd[0] + e.dd[2]);
     q[9 * stride] = e.d0 + (e.dd[1] + e.dd[2]);
 }
+// the same values in an array of registers (slot k at q[k]): the bulk-staged
+// kernel, whose shared memory holds tiles instead.  zero: -0, which the compiler
+// does not know, so that the products ab, db and dk round once here, as they do
+// on their way to shared memory, and are not fused into the sums that use them.
+__device__ __forceinline__ void hold_eq(const W2 &e, f2 (&q)[kEqSlots], f2 zero)
+{
+    park_eq(e, q, 1);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        q[4 + j] = q[4 + j] + zero;
+        q[10 + j] = q[10 + j] + zero;
+        q[13 + j] = q[13 + j] + zero;
+    }
+}
 template <int I>
 __device__ __forceinline__ f2 eq_parked(const f2 *q, int stride)
 {
@@ -678,22 +692,25 @@ struct BulkIO : PlaneIO {
 //
 // park (viscous step): this thread's slots in shared memory, slot k at
 // park[k * pstride]: the h-equilibrium coefficients wait there while the f
-// populations are updated (kParkH slots), and with PARKF the coefficients in
+// populations are updated (kParkH slots), and with EQ_PARKED the coefficients in
 // use too (kEqSlots more), which leaves their registers to the stencils in
-// flight.  Grids of 2 and 3 dimensions take PARKF (3-D: 3.58 ms a step with
+// flight.  Grids of 2 and 3 dimensions take EQ_PARKED (3-D: 3.58 ms a step with
 // three items in flight; with the f coefficients in registers one item fits,
-// 4.15 ms); in one dimension an item is three pairs and registers suffice.
+// 4.15 ms); in one dimension an item is three pairs and registers suffice
+// (EQ_FOLD).  EQ_HELD: the bulk-staged kernel (hold_eq).
 //
 // NP = 7 or 14: the 1-D or 2-D symmetry reduction (see rep and mult); only
 // the class representatives are read and written, and the previous level's
 // zero sums (sum c_z f; 1-D also sum c_y f) are left alone.
-template <bool EULER, bool PARKF, int NP, int LAT, bool REC64, typename IO>
+enum { EQ_FOLD, EQ_PARKED, EQ_HELD };
+template <bool EULER, int EQ, int NP, int LAT, bool REC64, typename IO>
 __device__ __forceinline__ void update_pair(const StepParams &p, IO &io, bool has1, float eos, f2 *park = nullptr,
                                             int pstride = 0)
 {
     static_assert(NP == 19 || !EULER, "the symmetry reductions are viscous");
     static_assert(!REC64 || (!EULER && NP == 19), "the FP64 recovery is a variant of the viscous 19-population step");
     io.begin();
+    const f2 zero = bc(__uint_as_float(0x80000000u | (unsigned(p.nx) >> 31)));   // see hold_eq
 
     if constexpr (!EULER) {
         // raw sums of the local populations: S = sum f, V_a = sum c_a f
@@ -799,7 +816,7 @@ __device__ __forceinline__ void update_pair(const StepParams &p, IO &io, bool ha
             if constexpr (has_vy<NP>()) io.template put_prev<2>(Vy.hi + Vy.lo);
             if constexpr (has_vz<NP>()) io.template put_prev<3>(Vz.hi + Vz.lo);
             io.template put_prev<4>(Sh);
-            f2 *hp = park + (PARKF ? kEqSlots * pstride : 0);
+            f2 *hp = park + (EQ == EQ_PARKED ? kEqSlots * pstride : 0);
             hp[0] = H0;
             hp[10 * pstride] = T0h;
 #pragma unroll
@@ -808,18 +825,21 @@ __device__ __forceinline__ void update_pair(const StepParams &p, IO &io, bool ha
                 hp[(4 + j) * pstride] = Hd[j];
                 hp[(7 + j) * pstride] = Ho[j];
             }
-            if constexpr (PARKF) park_eq(ef, park, pstride);
+            f2 held[kEqSlots];
+            if constexpr (EQ == EQ_PARKED) park_eq(ef, park, pstride);
+            if constexpr (EQ == EQ_HELD) hold_eq(ef, held, zero);
             for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 const f2 pre = io.template pre<k, k>();
                 f2 q;
-                if constexpr (PARKF) q = eq_parked<rep<NP>(k)>(park, pstride);
+                if constexpr (EQ == EQ_PARKED) q = eq_parked<rep<NP>(k)>(park, pstride);
+                else if constexpr (EQ == EQ_HELD) q = eq_parked<rep<NP>(k)>(held, 1);
                 else q = eq2<rep<NP>(k)>(ef);
                 io.template put<k>(fma2(kap, q - pre, pre));
             });
         }
         {
-            const f2 *hp = park + (PARKF ? kEqSlots * pstride : 0);
+            const f2 *hp = park + (EQ == EQ_PARKED ? kEqSlots * pstride : 0);
             H0 = hp[0];
             T0h = hp[10 * pstride];
 #pragma unroll
@@ -829,12 +849,15 @@ __device__ __forceinline__ void update_pair(const StepParams &p, IO &io, bool ha
                 Ho[j] = hp[(7 + j) * pstride];
             }
             const W2 eh = weigh2<Lat<LAT>::dmag>(H0, Hb, Hd, Ho, float(Lat<LAT>::wh0), float(Lat<LAT>::wh1), float(Lat<LAT>::wh2), T0h, nullptr);
-            if constexpr (PARKF) park_eq(eh, park, pstride);
+            f2 held[kEqSlots];
+            if constexpr (EQ == EQ_PARKED) park_eq(eh, park, pstride);
+            if constexpr (EQ == EQ_HELD) hold_eq(eh, held, zero);
             for_pops(std::make_integer_sequence<int, NP>{}, [&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 const f2 pre = io.template pre<NP + k, NP + k>();
                 f2 q;
-                if constexpr (PARKF) q = eq_parked<rep<NP>(k)>(park, pstride);
+                if constexpr (EQ == EQ_PARKED) q = eq_parked<rep<NP>(k)>(park, pstride);
+                else if constexpr (EQ == EQ_HELD) q = eq_parked<rep<NP>(k)>(held, 1);
                 else q = eq2<rep<NP>(k)>(eh);
                 io.template put<NP + k>(fma2(kap, q - pre, pre));
             });
@@ -990,7 +1013,7 @@ __global__ void __launch_bounds__(32 * RLB_F32_BY, RLB_F32_MINB)
     // sit at fixed offsets from one base address
     constexpr int nthr = (DIM == 1 && !LIN) ? kTubeThreads : 32 * RLB_F32_BY;
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    update_pair<EULER, (DIM > 1), NP, LAT, REC64>(p, io, has1, p.f_eta_over_s, s_park + tid, nthr);
+    update_pair<EULER, (DIM > 1) ? EQ_PARKED : EQ_FOLD, NP, LAT, REC64>(p, io, has1, p.f_eta_over_s, s_park + tid, nthr);
 }
 
 }  // namespace f32

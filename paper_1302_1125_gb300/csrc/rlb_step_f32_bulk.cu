@@ -18,7 +18,7 @@ constexpr int kBulkThreads = 256;   // 32 x 8
 // the row and plane maps
 constexpr size_t bulk_smem_bytes()
 {
-    return sizeof(float) * size_t(kBulkBufs) * kTileFloats + sizeof(f2) * size_t(kParkH + kEqSlots) * kBulkThreads +
+    return sizeof(float) * size_t(kBulkBufs) * kTileFloats + sizeof(f2) * size_t(kParkH) * kBulkThreads +
            sizeof(unsigned long long) * kBulkBufs + 2 * sizeof(int) * kBulkBufs + sizeof(int) * 16;
 }
 
@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(kBulkThreads, 2)
     float *tiles = reinterpret_cast<float *>(smem);
     f2 *park = reinterpret_cast<f2 *>(smem + sizeof(float) * size_t(kBulkBufs) * kTileFloats);
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(
-        smem + sizeof(float) * size_t(kBulkBufs) * kTileFloats + sizeof(f2) * size_t(kParkH + kEqSlots) * kBulkThreads);
+        smem + sizeof(float) * size_t(kBulkBufs) * kTileFloats + sizeof(f2) * size_t(kParkH) * kBulkThreads);
     int *issued = reinterpret_cast<int *>(bars + kBulkBufs);
     int *done = issued + kBulkBufs;
     int *ymap = done + kBulkBufs, *zmap = ymap + 12;
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kBulkThreads, 2)
     BulkIO<LAT> io{{p, f, h, fo, ho, prev, p.ps, x0 + p.nx * (y + p.ny * z), 0u, p.f_kbulk}, &b};
     if (x0 == 0) io.xfix |= p.bc_lo[0] == BC_OUTFLOW ? XF_LO_CLAMP : XF_LO_GHOST;
     if (x0 + 2 >= p.nx) io.xfix |= p.bc_hi[0] == BC_OUTFLOW ? XF_HI_CLAMP : XF_HI_GHOST;
-    update_pair<false, true, 19, LAT, false>(p, io, true, p.f_eta_over_s, park + tid, kBulkThreads);
+    update_pair<false, EQ_HELD, 19, LAT, false>(p, io, true, p.f_eta_over_s, park + tid, kBulkThreads);
 
     // after a timeout: let the copies this block issued land before the
     // shared memory is released (bounded as well)
