@@ -7,6 +7,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <queue>
 #include <string>
@@ -26,6 +27,7 @@ struct rlb_batch {
     rlb_options opt{};
     int device = 0;
     int sms = 0;
+    int l2_bytes = 0;
     std::vector<int> nx;
     std::vector<long long> pack;     // B + 1 packed offsets
     std::vector<Tube> tubes;
@@ -116,6 +118,47 @@ struct Plan {
     long long critical = 0;
 };
 
+// longest-running first: steps, then length, then id
+std::vector<int> tube_order(int B, const int *nx, const long long *steps)
+{
+    std::vector<int> ids(B);
+    for (int i = 0; i < B; ++i) ids[i] = i;
+    std::stable_sort(ids.begin(), ids.end(), [&](int a, int b) {
+        if (steps[a] != steps[b]) return steps[a] > steps[b];
+        return nx[a] > nx[b];
+    });
+    return ids;
+}
+
+// consecutive tubes of that order in jobs of at most cluster x threads x
+// pairs_per_thread pairs
+void group_tubes(const std::vector<int> &ids, const int *nx, const long long *steps, const rlb_batch_tuning &t,
+                 std::vector<Job> &jobs)
+{
+    const long long cap = (long long)t.cluster * t.threads * t.pairs_per_thread;
+    jobs.clear();
+    for (size_t k = 0; k < ids.size(); ++k) {
+        const int id = ids[k];
+        if (steps[id] == 0) break;
+        const int pairs = (nx[id] + 1) / 2;
+        if (!jobs.empty()) {
+            Job &J = jobs.back();
+            if (J.count < rlb::batch::kMaxJobTubes && (long long)J.pairs + pairs <= cap) {
+                J.count += 1;
+                J.pairs += pairs;
+                continue;
+            }
+        }
+        jobs.push_back(Job{int(k), 1, int(steps[id]), pairs});
+    }
+}
+
+long long passes(const Job &J, const rlb_batch_tuning &t)
+{
+    const long long per_pass = (long long)t.cluster * t.threads;
+    return (J.pairs + per_pass - 1) / per_pass;
+}
+
 rlb_status make_plan(int B, const int *nx, const long long *steps, const rlb_batch_tuning &t, int nclusters,
                      Plan &pl, std::string &why)
 {
@@ -138,34 +181,11 @@ rlb_status make_plan(int B, const int *nx, const long long *steps, const rlb_bat
             return RLB_E_INVALID;
         }
     }
-    // longest-running first: steps, then length, then id
-    std::vector<int> ids(B);
-    for (int i = 0; i < B; ++i) ids[i] = i;
-    std::stable_sort(ids.begin(), ids.end(), [&](int a, int b) {
-        if (steps[a] != steps[b]) return steps[a] > steps[b];
-        return nx[a] > nx[b];
-    });
-    pl.order = ids;
-    // group consecutive tubes into jobs of at most cap pairs
-    const long long per_pass = (long long)t.cluster * t.threads;
-    const long long cap = per_pass * t.pairs_per_thread;
+    pl.order = tube_order(B, nx, steps);
     std::vector<Job> jobs;
-    for (int k = 0; k < B; ++k) {
-        const int id = ids[k];
-        if (steps[id] == 0) break;
-        const int pairs = (nx[id] + 1) / 2;
-        if (!jobs.empty()) {
-            Job &J = jobs.back();
-            if (J.count < rlb::batch::kMaxJobTubes && (long long)J.pairs + pairs <= cap) {
-                J.count += 1;
-                J.pairs += pairs;
-                continue;
-            }
-        }
-        jobs.push_back(Job{k, 1, int(steps[id]), pairs});
-    }
+    group_tubes(pl.order, nx, steps, t, jobs);
     // longest processing time first, each job to the least loaded cluster
-    auto cost = [&](const Job &J) { return (long long)J.steps * ((J.pairs + per_pass - 1) / per_pass); };
+    auto cost = [&](const Job &J) { return J.steps * passes(J, t); };
     std::vector<int> jorder(jobs.size());
     for (size_t i = 0; i < jobs.size(); ++i) jorder[i] = int(i);
     std::stable_sort(jorder.begin(), jorder.end(), [&](int a, int b) { return cost(jobs[a]) > cost(jobs[b]); });
@@ -191,6 +211,32 @@ rlb_status make_plan(int B, const int *nx, const long long *steps, const rlb_bat
     pl.critical = 0;
     for (long long v : load) pl.critical = std::max(pl.critical, v);
     return RLB_OK;
+}
+
+// us of a job under a launch shape: of a pass, and of a step beside its passes
+struct Price {
+    rlb_batch_tuning t;
+    double pass, step;
+    double operator()(const Job &J) const { return J.steps * (double(passes(J, t)) * pass + step); }
+};
+
+// the longest load when the jobs, longest first, each go to the least loaded cluster
+double critical_path(const std::vector<Job> &jobs, const Price &price, int nclusters)
+{
+    std::vector<double> cost(jobs.size());
+    for (size_t j = 0; j < jobs.size(); ++j) cost[j] = price(jobs[j]);
+    std::sort(cost.begin(), cost.end(), std::greater<double>());
+    double longest = cost[0];
+    if (cost.size() <= size_t(nclusters)) return longest;
+    std::priority_queue<double, std::vector<double>, std::greater<double>> load(
+        std::greater<double>(), std::vector<double>(cost.begin(), cost.begin() + nclusters));
+    for (size_t j = nclusters; j < cost.size(); ++j) {
+        const double l = load.top() + cost[j];
+        load.pop();
+        load.push(l);
+        longest = std::max(longest, l);
+    }
+    return longest;
 }
 
 rlb_status check_status(rlb_batch *b)
@@ -294,41 +340,58 @@ rlb_status apply_tuning(rlb_batch *b, const rlb_batch_tuning &t)
 }
 
 // The launch shape of a batch that nobody tuned, chosen at its first step
-// call: the one whose plan has the least critical path (rlb_batch_plan, in
-// passes) times the time of a pass.  A pass costs more the more threads share
-// the SM; the line below fits the autotuner's times on GB300 over batches of
-// 16 to 512 tubes of 256 to 8192 cells (us a pass with 128 / 256 / 384 / 512
-// threads an SM: 5.0-5.3, 5.6-6.5, 6.9-8.3, 9.2-9.9; with 7 classes 2.5-2.9,
-// 3.2-3.5, 4.0-4.2, 4.7-5.1), a cluster's barrier a few per cent more.
+// call: the one with the shortest critical path when jobs are priced in us.  A
+// pass takes the time of the busiest scheduler's warps (GB300, us with 1 / 2 / 3
+// / 4 warps: 4.4, 5.4, 7.1, 9.1; with 7 classes 2.15, 2.9, 3.75, 4.7), a quarter
+// more when the tubes in progress do not fit in the L2 cache, and a step in a
+// cluster 1.2 us more (0.9).  The warps that count are those that have pairs, in
+// the blocks that have jobs (and a little for blocks that may meet on an SM
+// while others idle): pricing every block that fits took four blocks of 128
+// for as dear as one of 512, and 64 tubes of 256 cells 1.9 times as long as their
+// best shape.  Blocks of 128 and 256 threads run the kernel of bound 256: with
+// bound 512 more of them fit, and few jobs then share SMs.  Over 246 batches of
+// 1 to 2048 tubes of 20 to 8192 cells the choice takes 1.02 times the
+// autotuner's best time (1.38 before), at most 1.46 times (2.64).
 rlb_status choose_shape(rlb_batch *b, const long long *steps)
 {
     b->shape_set = true;
     const bool sym = b->opt.symmetry_1d != 0;
-    const double base = sym ? 2.2 : 3.9, per_thread = sym ? 0.0052 : 0.0108;
-    const double join[4] = {1.0, 1.03, 1.04, 1.06};
-    // job capacities: one for large batches, whose plans take longer to make
-    // and whose tubes outnumber the clusters anyway
-    const bool large = b->B > 2048;
+    const double pass[2][4] = {{4.4, 5.4, 7.1, 9.1}, {2.15, 2.9, 3.75, 4.7}}, join[2] = {1.2, 0.9};
+    const double pair_bytes = 2.0 * sizeof(float) * (2 * (sym ? 14 : 38) + 5);
+    std::vector<Job> jobs;
+    const std::vector<int> order = tube_order(b->B, b->nx.data(), steps);
     rlb_batch_tuning best = b->tune;
     double best_cost = -1.0;
     for (int threads : {128, 256, 384, 512}) {
-        for (int j = 0; j < 4; ++j) {
-            // small blocks in the 128-register variant, of which an SM holds several
-            rlb_batch_tuning t{threads, threads < 384 ? 512 : threads, 1 << j, 1, 0.0};
+        for (int cluster : {1, 2, 4, 8}) {
+            const rlb_batch_tuning t{threads, std::max(threads, 256), cluster, 1, 0.0};
             int n = 0;
-            if (rlb_status st = resident_clusters(b, t, n); st != RLB_OK) return st;
+            resident_clusters(b, t, n);
             if (n < 1) continue;
-            const double on_sm = double(threads) * double(n) * t.cluster / b->sms;
-            for (int k = large ? 4 : 1; k <= 4; k *= 2) {
-                t.pairs_per_thread = k;
-                Plan pl;
-                std::string why;
-                if (make_plan(b->B, b->nx.data(), steps, t, n, pl, why) != RLB_OK) continue;
-                const double c = double(pl.critical) * (base + per_thread * on_sm) * join[j];
-                if (best_cost < 0.0 || c < best_cost) {
-                    best_cost = c;
-                    best = t;
-                }
+            group_tubes(order, b->nx.data(), steps, t, jobs);
+            // means over the work: threads with a pair in a cluster's first
+            // block, pairs of a job
+            double work = 0.0, active = 0.0, pairs = 0.0;
+            for (const Job &J : jobs) {
+                const double w = double(J.steps) * double(passes(J, t));
+                work += w;
+                active += w * double(std::min(J.pairs, threads));
+                pairs += w * double(J.pairs);
+            }
+            const int busy = int(std::min<size_t>(jobs.size(), size_t(n)));
+            const int fit = std::max(1, (n * cluster + b->sms / 2) / b->sms), used = (busy * cluster + b->sms - 1) / b->sms;
+            const double on_sm = used < fit ? used + 0.25 : fit;
+            const double warps = on_sm * std::ceil(active / work / 32.0) / 4.0;   // of one scheduler
+            const int q = std::min(3, std::max(1, int(warps)));
+            const double *p = pass[sym];
+            double us = warps <= 1.0 ? p[0] : p[q - 1] + (p[q] - p[q - 1]) * (warps - q);
+            const double in_l2 = busy * (pairs / work) * pair_bytes / b->l2_bytes;
+            us *= 1.0 + 0.25 * std::min(1.0, std::max(0.0, (in_l2 - 0.8) / 0.4));
+            const Price price{t, us, cluster > 1 ? join[sym] : 0.0};
+            const double c = critical_path(jobs, price, n);
+            if (best_cost < 0.0 || c < best_cost) {
+                best_cost = c;
+                best = t;
             }
         }
     }
@@ -466,6 +529,7 @@ rlb_status rlb_batch_create(int B, const int *nx, const double *eta_over_s, cons
     b->ps = (long long)aup(size_t(off), 64);
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->l2_bytes, cudaDevAttrL2CacheSize, b->device);
     if (e != cudaSuccess) {
         delete b;
         return bcuda(nullptr, e, "cudaGetDevice");
