@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
+#include <mutex>
 #include <new>
 #include <queue>
 #include <string>
@@ -285,6 +286,28 @@ rlb_status resident_clusters(rlb_batch *b, const rlb_batch_tuning &t, int &n)
     return RLB_OK;
 }
 
+// The same for the shapes choose_shape looks at, asked once per process for
+// each device and form: it depends on the kernels alone.
+int resident_shape(rlb_batch *b, const rlb_batch_tuning &t)
+{
+    constexpr int kMaxDevices = 64;
+    static std::mutex lock;
+    static int known[kMaxDevices][2][4][4];   // 0: not asked yet, else clusters + 1
+    int n = 0;
+    if (b->device >= kMaxDevices) {
+        resident_clusters(b, t, n);
+        return n;
+    }
+    const std::lock_guard<std::mutex> hold(lock);
+    const int j = t.cluster == 8 ? 3 : t.cluster / 2;
+    int &k = known[b->device][b->opt.symmetry_1d != 0][t.threads / 128 - 1][j];
+    if (k == 0) {
+        resident_clusters(b, t, n);
+        k = n + 1;
+    }
+    return std::min(k - 1, b->max_clusters);
+}
+
 rlb_status upload_plan(rlb_batch *b, const long long *steps, const Plan &pl)
 {
     for (int i = 0; i < b->B; ++i) b->h_steps[i] = int(steps[i]);
@@ -352,21 +375,28 @@ rlb_status apply_tuning(rlb_batch *b, const rlb_batch_tuning &t)
 // bound 512 more of them fit, and few jobs then share SMs.  Over 246 batches of
 // 1 to 2048 tubes of 20 to 8192 cells the choice takes 1.02 times the
 // autotuner's best time (1.38 before), at most 1.46 times (2.64).
+//
+// The tubes are sorted once, and a shape's jobs are laid out only while its lower
+// bound (the longest job, or all work over all clusters) is below the best
+// critical path so far.
 rlb_status choose_shape(rlb_batch *b, const long long *steps)
 {
     b->shape_set = true;
     const bool sym = b->opt.symmetry_1d != 0;
     const double pass[2][4] = {{4.4, 5.4, 7.1, 9.1}, {2.15, 2.9, 3.75, 4.7}}, join[2] = {1.2, 0.9};
     const double pair_bytes = 2.0 * sizeof(float) * (2 * (sym ? 14 : 38) + 5);
+    struct Shape {
+        Price price;
+        int n;
+        double bound;   // of the critical path
+    };
+    std::vector<Shape> shapes;
     std::vector<Job> jobs;
     const std::vector<int> order = tube_order(b->B, b->nx.data(), steps);
-    rlb_batch_tuning best = b->tune;
-    double best_cost = -1.0;
     for (int threads : {128, 256, 384, 512}) {
         for (int cluster : {1, 2, 4, 8}) {
             const rlb_batch_tuning t{threads, std::max(threads, 256), cluster, 1, 0.0};
-            int n = 0;
-            resident_clusters(b, t, n);
+            const int n = resident_shape(b, t);
             if (n < 1) continue;
             group_tubes(order, b->nx.data(), steps, t, jobs);
             // means over the work: threads with a pair in a cluster's first
@@ -388,14 +418,28 @@ rlb_status choose_shape(rlb_batch *b, const long long *steps)
             const double in_l2 = busy * (pairs / work) * pair_bytes / b->l2_bytes;
             us *= 1.0 + 0.25 * std::min(1.0, std::max(0.0, (in_l2 - 0.8) / 0.4));
             const Price price{t, us, cluster > 1 ? join[sym] : 0.0};
-            const double c = critical_path(jobs, price, n);
-            if (best_cost < 0.0 || c < best_cost) {
-                best_cost = c;
-                best = t;
+            double longest = 0.0, total = 0.0;
+            for (const Job &J : jobs) {
+                const double c = price(J);
+                total += c;
+                longest = std::max(longest, c);
             }
+            shapes.push_back(Shape{price, n, std::max(longest, total / n)});
         }
     }
-    return best_cost < 0.0 ? RLB_OK : apply_tuning(b, best);
+    std::stable_sort(shapes.begin(), shapes.end(), [](const Shape &x, const Shape &y) { return x.bound < y.bound; });
+    const Shape *best = nullptr;
+    double best_cost = 0.0;
+    for (const Shape &s : shapes) {
+        if (best && s.bound >= best_cost) break;
+        group_tubes(order, b->nx.data(), steps, s.price.t, jobs);
+        const double c = critical_path(jobs, s.price, s.n);
+        if (!best || c < best_cost) {
+            best_cost = c;
+            best = &s;
+        }
+    }
+    return best ? apply_tuning(b, best->price.t) : RLB_OK;
 }
 
 rlb_status ensure_graph(rlb_batch *b)
