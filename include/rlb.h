@@ -395,9 +395,9 @@ RLB_API rlb_status rlb_batch_init(rlb_batch *b, const double *n, const double *T
  * [0, 2^31 - 1]; 0 leaves a tube unchanged) in one launch of the persistent
  * kernel, replayed from a CUDA graph.  The job plan is rebuilt when the step
  * counts or the tuning change.  Unless rlb_batch_set_tuning or
- * rlb_batch_autotune set a launch shape, the first call chooses one for its
- * step counts from the plans of several shapes and measured pass times, and
- * later calls keep it.  Waits for the launch and returns
+ * rlb_batch_autotune set a launch shape, each new plan chooses one for its
+ * step counts from the critical paths of several shapes at measured pass
+ * times.  Waits for the launch and returns
  * RLB_E_NONPHYSICAL if any cell of any step was non-physical. */
 RLB_API rlb_status rlb_batch_step(rlb_batch *b, const long long *nsteps);
 

@@ -53,7 +53,7 @@ struct rlb_batch {
     double *h_tot = nullptr;
     rlb_batch_tuning tune{};
     int nclusters = 0;               // clusters resident at once for `tune`
-    bool shape_set = false;          // the launch shape was set, tuned or chosen (choose_shape)
+    bool shape_set = false;          // the launch shape was set or tuned (else choose_shape's)
     bool plan_ok = false;
     std::vector<long long> plan_steps;
     cudaStream_t stream = nullptr, cap_stream = nullptr;
@@ -324,11 +324,16 @@ rlb_status upload_plan(rlb_batch *b, const long long *steps, const Plan &pl)
     return RLB_OK;
 }
 
+bool planned(const rlb_batch *b, const long long *steps)
+{
+    return b->plan_ok && std::equal(b->plan_steps.begin(), b->plan_steps.end(), steps);
+}
+
 // plan for `steps` under the current tuning, uploaded (the host staging is
 // reused only after the previous call synchronised)
 rlb_status prepare(rlb_batch *b, const long long *steps)
 {
-    if (b->plan_ok && std::equal(b->plan_steps.begin(), b->plan_steps.end(), steps)) return RLB_OK;
+    if (planned(b, steps)) return RLB_OK;
     Plan pl;
     std::string why;
     rlb_status st = make_plan(b->B, b->nx.data(), steps, b->tune, b->nclusters, pl, why);
@@ -362,8 +367,9 @@ rlb_status apply_tuning(rlb_batch *b, const rlb_batch_tuning &t)
     return RLB_OK;
 }
 
-// The launch shape of a batch that nobody tuned, chosen at its first step
-// call: the one with the shortest critical path when jobs are priced in us.  A
+// The launch shape of a batch that nobody tuned, chosen with each new plan (one
+// kept from a call that advanced a single tube made 512 tubes take twice as
+// long): the one with the shortest critical path when jobs are priced in us.  A
 // pass takes the time of the busiest scheduler's warps (GB300, us with 1 / 2 / 3
 // / 4 warps: 4.4, 5.4, 7.1, 9.1; with 7 classes 2.15, 2.9, 3.75, 4.7), a quarter
 // more when the tubes in progress do not fit in the L2 cache, and a step in a
@@ -381,7 +387,6 @@ rlb_status apply_tuning(rlb_batch *b, const rlb_batch_tuning &t)
 // critical path so far.
 rlb_status choose_shape(rlb_batch *b, const long long *steps)
 {
-    b->shape_set = true;
     const bool sym = b->opt.symmetry_1d != 0;
     const double pass[2][4] = {{4.4, 5.4, 7.1, 9.1}, {2.15, 2.9, 3.75, 4.7}}, join[2] = {1.2, 0.9};
     const double pair_bytes = 2.0 * sizeof(float) * (2 * (sym ? 14 : 38) + 5);
@@ -439,7 +444,12 @@ rlb_status choose_shape(rlb_batch *b, const long long *steps)
             best = &s;
         }
     }
-    return best ? apply_tuning(b, best->price.t) : RLB_OK;
+    if (!best) return RLB_OK;
+    const rlb_batch_tuning &t = best->price.t, &now = b->tune;
+    if (t.threads == now.threads && t.bound == now.bound && t.cluster == now.cluster &&
+        t.pairs_per_thread == now.pairs_per_thread)
+        return RLB_OK;
+    return apply_tuning(b, t);
 }
 
 rlb_status ensure_graph(rlb_batch *b)
@@ -663,8 +673,8 @@ rlb_status rlb_batch_create(int B, const int *nx, const double *eta_over_s, cons
     sp.f_kw = float(sp.kw);
     sp.f_tau_override = float(sp.tau_override);
 
-    // a shape that fits every GB300 configuration, until the first step call
-    // chooses one for its step counts; rlb_batch_autotune measures them
+    // a shape that fits every GB300 configuration, until a step call chooses one
+    // for its step counts; rlb_batch_autotune measures them
     rlb_batch_tuning t{256, 256, 1, 1, 0.0};
     const rlb_status st = apply_tuning(b, t);
     if (st != RLB_OK) {
@@ -707,7 +717,7 @@ rlb_status rlb_batch_step(rlb_batch *b, const long long *nsteps)
     for (int i = 0; i < b->B; ++i) any = any || nsteps[i] > 0;
     if (!any) return RLB_OK;
     RLB_BCUDA(b, cudaSetDevice(b->device));
-    if (!b->shape_set && (st = choose_shape(b, nsteps)) != RLB_OK) return st;
+    if (!b->shape_set && !planned(b, nsteps) && (st = choose_shape(b, nsteps)) != RLB_OK) return st;
     if ((st = prepare(b, nsteps)) != RLB_OK) return st;
     if ((st = ensure_graph(b)) != RLB_OK) return st;
     RLB_BCUDA(b, cudaGraphLaunch(b->graph, b->stream));

@@ -74,3 +74,33 @@ def test_the_choice_costs_little_of_the_first_call():
         extra.append((t1 - t0) - (time.perf_counter() - t1))
         b.close()
     assert min(extra) < 1.0e-3
+
+
+def test_the_shape_follows_the_step_counts():
+    """a call that advances one tube, or a few steps, leaves no shape behind;
+    the results do not depend on the shape"""
+    rng = np.random.default_rng(2)
+    nx = np.exp(rng.uniform(np.log(256), np.log(8192), 200)).astype(np.int32)
+    one, steps = np.zeros(200, np.int64), (nx // 64).astype(np.int64)
+    one[7] = 3
+    fresh, other = batch(nx).step(steps), batch(nx).step(one)
+    assert shape(other) != shape(fresh)
+    other.step(steps)
+    assert shape(other) == shape(fresh)
+    fresh.step(one)
+    assert shape(fresh) != shape(other)
+    a, c = fresh.macroscopic(device=False), other.macroscopic(device=False)
+    keep = np.ones(fresh.total, bool)
+    keep[fresh.offsets[7]:fresh.offsets[8]] = False      # tube 7 took its steps in another order: alike too
+    assert np.array_equal(a[:, keep], c[:, keep]) and np.array_equal(a, c)
+
+
+def test_a_shape_set_by_hand_or_tuned_stays():
+    nx = np.array([300, 64, 5000, 128], np.int32)
+    b = batch(nx)
+    b.set_tuning(64, 512, 2, 2)
+    b.step(8).step([1, 0, 0, 0])
+    assert shape(b) == (64, 512, 2, 2)
+    best, _ = b.autotune(8, divisor=1)
+    b.step(8).step([0, 0, 9, 1])
+    assert shape(b) == (best.threads, best.bound, best.cluster, best.pairs_per_thread)
