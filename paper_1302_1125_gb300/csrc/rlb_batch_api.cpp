@@ -214,11 +214,16 @@ rlb_status make_plan(int B, const int *nx, const long long *steps, const rlb_bat
     return RLB_OK;
 }
 
-// us of a job under a launch shape: of a pass, and of a step beside its passes
+// us of a job under a launch shape: passes in which w warps of a cluster's first
+// block have pairs take us[w] each, a step `step` more
 struct Price {
     rlb_batch_tuning t;
-    double pass, step;
-    double operator()(const Job &J) const { return J.steps * (double(passes(J, t)) * pass + step); }
+    double us[17], step;
+    double operator()(const Job &J) const
+    {
+        const int per_pass = t.cluster * t.threads, full = J.pairs / per_pass, rest = J.pairs - full * per_pass;
+        return J.steps * (full * us[t.threads / 32] + us[(std::min(rest, t.threads) + 31) / 32] + step);
+    }
 };
 
 // the longest load when the jobs, longest first, each go to the least loaded cluster
@@ -371,15 +376,15 @@ rlb_status apply_tuning(rlb_batch *b, const rlb_batch_tuning &t)
 // kept from a call that advanced a single tube made 512 tubes take twice as
 // long): the one with the shortest critical path when jobs are priced in us.  A
 // pass takes the time of the busiest scheduler's warps (GB300, us with 1 / 2 / 3
-// / 4 warps: 4.4, 5.4, 7.1, 9.1; with 7 classes 2.15, 2.9, 3.75, 4.7), a quarter
-// more when the tubes in progress do not fit in the L2 cache, and a step in a
-// cluster 1.2 us more (0.9).  The warps that count are those that have pairs, in
-// the blocks that have jobs (and a little for blocks that may meet on an SM
-// while others idle): pricing every block that fits took four blocks of 128
-// for as dear as one of 512, and 64 tubes of 256 cells 1.9 times as long as their
-// best shape.  Blocks of 128 and 256 threads run the kernel of bound 256: with
-// bound 512 more of them fit, and few jobs then share SMs.  Over 246 batches of
-// 1 to 2048 tubes of 20 to 8192 cells the choice takes 1.02 times the
+// / 4 warps: 4.4, 5.4, 7.1, 9.1; with 7 classes 2.15, 2.9, 3.75, 4.7), up to a
+// third more when the tubes in progress do not fit in the L2 cache, and a step
+// in a cluster 1.2 us more (0.9).  The warps that count are those that have
+// pairs, in the blocks that have jobs (and a little for blocks that may meet on
+// an SM while others idle): pricing every block that fits took four blocks of
+// 128 for as dear as one of 512, and 64 tubes of 256 cells 1.9 times as long as
+// their best shape.  Blocks of 128 and 256 threads run the kernel of bound 256:
+// with bound 512 more of them fit, and few jobs then share SMs.  Over 246 batches
+// of 1 to 2048 tubes of 20 to 8192 cells the choice takes 1.03 times the
 // autotuner's best time (1.38 before), at most 1.46 times (2.64).
 //
 // The tubes are sorted once, and a shape's jobs are laid out only while its lower
@@ -404,25 +409,24 @@ rlb_status choose_shape(rlb_batch *b, const long long *steps)
             const int n = resident_shape(b, t);
             if (n < 1) continue;
             group_tubes(order, b->nx.data(), steps, t, jobs);
-            // means over the work: threads with a pair in a cluster's first
-            // block, pairs of a job
-            double work = 0.0, active = 0.0, pairs = 0.0;
+            double work = 0.0, pairs = 0.0;   // pairs of a job, mean over the work
             for (const Job &J : jobs) {
                 const double w = double(J.steps) * double(passes(J, t));
                 work += w;
-                active += w * double(std::min(J.pairs, threads));
                 pairs += w * double(J.pairs);
             }
             const int busy = int(std::min<size_t>(jobs.size(), size_t(n)));
             const int fit = std::max(1, (n * cluster + b->sms / 2) / b->sms), used = (busy * cluster + b->sms - 1) / b->sms;
             const double on_sm = used < fit ? used + 0.25 : fit;
-            const double warps = on_sm * std::ceil(active / work / 32.0) / 4.0;   // of one scheduler
-            const int q = std::min(3, std::max(1, int(warps)));
-            const double *p = pass[sym];
-            double us = warps <= 1.0 ? p[0] : p[q - 1] + (p[q] - p[q - 1]) * (warps - q);
             const double in_l2 = busy * (pairs / work) * pair_bytes / b->l2_bytes;
-            us *= 1.0 + 0.25 * std::min(1.0, std::max(0.0, (in_l2 - 0.8) / 0.4));
-            const Price price{t, us, cluster > 1 ? join[sym] : 0.0};
+            const double far = 1.0 + 0.35 * std::max(0.0, 1.0 - 0.8 / in_l2);
+            Price price{t, {0.0}, cluster > 1 ? join[sym] : 0.0};
+            for (int w = 1; w <= threads / 32; ++w) {
+                const double warps = on_sm * w / 4.0;   // of one scheduler
+                const int q = std::min(3, std::max(1, int(warps)));
+                const double *p = pass[sym];
+                price.us[w] = far * (warps <= 1.0 ? p[0] : p[q - 1] + (p[q] - p[q - 1]) * (warps - q));
+            }
             double longest = 0.0, total = 0.0;
             for (const Job &J : jobs) {
                 const double c = price(J);
