@@ -111,7 +111,8 @@ __device__ __noinline__ double streamed_called(const Sten64 q, double qc, double
 // step about twice as long, and a kernel with a warp or two per scheduler waits
 // for instructions: the four-warp kernel (step_split_kernel) takes 22 us a step
 // on 64 x 64 cells inlined, 18.2 called, and in 3-D 151 registers, with which a
-// fourth block does not fit on an SM (32 x 32 x 18 cells 64 us), or 126 (34 us).
+// fourth block does not fit on an SM (32 x 32 x 18 cells 64 us), or 126 (34 us);
+// tiles with a block or less an SM 58.4 us on 16 x 16 x 8 cells, 50.6 called.
 // With four warps per scheduler the call costs more than it saves (1024 x 512
 // cells 690 us inlined, 756 called), but not in Euler mode, whose streaming is
 // all in one loop (64 x 64 cells 34.7 and 27.4, 256 x 128 x 128 5080 and 4310).

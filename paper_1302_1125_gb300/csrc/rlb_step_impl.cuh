@@ -71,6 +71,12 @@ cudaError_t launch_step_np(const StepParams &p, const T *f, const T *h, T *fo, T
             return launch_overlapped(step_kernel<T, DIM, EULER, LAT, true, NP>, nb, bs, 0, s, p, f, h, fo, ho, prev);
         } else {
             const dim3 grid(unsigned(tiles_x), unsigned(tiles_y), p.nz);
+            // (a block or less an SM: see FX_CALL)
+            if constexpr (!EULER) {
+                if (f64_below(p, 128))
+                    return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP, FX_CALL>, grid, dim3(32, 4, 1), 0, s,
+                                             p, f, h, fo, ho, prev);
+            }
             return launch_overlapped(step_kernel<T, DIM, EULER, LAT, false, NP>, grid, dim3(32, 4, 1), 0, s, p, f, h, fo,
                                      ho, prev);
         }
