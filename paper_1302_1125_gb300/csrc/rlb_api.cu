@@ -1,5 +1,6 @@
 // rlb_api.cu -- the C ABI of librlb (declared in include/rlb.h): argument
 // validation, device memory of a context, and the host side of every call.
+#include <cudaTypedefs.h>   // PFN_cuPointerGetAttribute
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -547,15 +548,36 @@ size_t rlb_state_bytes(const rlb_ctx *ctx)
     return ctx ? (size_t)43 * ctx->N * ctx->esize : 0;
 }
 
+// whether the bytes at p, an address the device can use, lie in one allocation
+static bool in_one_allocation(const void *p, size_t bytes)
+{
+    static const PFN_cuPointerGetAttribute_v4000 attribute = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 4000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(fn);
+    }();
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    return attribute && attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) == CUDA_SUCCESS &&
+           attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) == CUDA_SUCCESS && rlb::holds(start, size, at, bytes);
+}
+
 // the blocks of the FP32 form as compact planes (38 populations, then 5
 // previous-level values) at buf: a device buffer of this GPU directly, any
-// other through the idle population buffer (38 planes of at least N)
+// other through the idle population buffer (38 planes of at least N).  A device
+// buffer that ends before the state does is not written by a kernel: it takes
+// the other way, where the copy refuses it.
 static rlb_status copy_blocks(rlb_ctx *ctx, void *buf, bool out)
 {
     cudaPointerAttributes at;
     const bool known = cudaPointerGetAttributes(&at, buf) == cudaSuccess;
     if (!known) cudaGetLastError();
-    const bool direct = known && at.type == cudaMemoryTypeDevice && at.device == ctx->device && (size_t)buf % 4 == 0;
+    const bool direct = known && at.type == cudaMemoryTypeDevice && at.device == ctx->device && (size_t)buf % 4 == 0 &&
+                        in_one_allocation(buf, rlb_state_bytes(ctx));
     char *user = (char *)buf;
     for (int k : {38, 5}) {
         float *blocks = (float *)(k == 38 ? ctx->fbuf[ctx->cur] : ctx->prev);

@@ -53,6 +53,12 @@ cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_
     return e;
 }
 
+// whether the allocation of `size` bytes at `start` holds `bytes` bytes from `at`
+inline bool holds(unsigned long long start, size_t size, unsigned long long at, size_t bytes)
+{
+    return at >= start && at - start <= size && bytes <= size - (at - start);
+}
+
 // Storage of a grid's populations: planes of stride ps (FP64 form; FP32 grids
 // staged by bulk copies), or blocks of 32 cells (the other FP32 grids,
 // rlb_step_f32.cuh)
