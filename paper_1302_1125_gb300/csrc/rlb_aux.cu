@@ -126,13 +126,14 @@ __global__ void solid_reset_kernel_f32(int M, const int *__restrict__ idx, f32::
 }
 
 // blocks <-> compact planes of N (rlb_get_state, rlb_set_state): K values of
-// each cell, value k of block cell i at src[at + 32 k]
-template <bool OUT, int K>
+// each cell (PREV: of the previous level), value k of block cell i at
+// blocks[at + 32 k]
+template <bool OUT, int K, bool PREV>
 __global__ void state_kernel(int N, f32::Store st, float *__restrict__ blocks, float *__restrict__ planes)
 {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
-    const long long i = st.cell(c), a = K == 5 ? st.prev_at(i) : st.at(i);
+    const long long i = st.cell(c), a = PREV ? st.prev_at(i) : st.at(i);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         if constexpr (OUT) planes[(long long)k * N + c] = blocks[a + k * f32::kBlk];
@@ -215,18 +216,26 @@ cudaError_t launch_sym(int fp32, int expand, int sym, int N, const Layout &l, vo
     return cudaGetLastError();
 }
 
-cudaError_t launch_state(bool out, int N, const Layout &l, int k, float *blocks, float *planes, cudaStream_t s)
+cudaError_t launch_state(bool out, int N, const Layout &l, StatePart part, float *blocks, float *planes, cudaStream_t s)
 {
     const int b = 256, g = (N + b - 1) / b;
-    const f32::Store st = store_of(l);
-    if (k == 5) {
-        if (out) state_kernel<true, 5><<<g, b, 0, s>>>(N, st, blocks, planes);
-        else state_kernel<false, 5><<<g, b, 0, s>>>(N, st, blocks, planes);
-    } else if (k == 38) {
-        if (out) state_kernel<true, 38><<<g, b, 0, s>>>(N, st, blocks, planes);
-        else state_kernel<false, 38><<<g, b, 0, s>>>(N, st, blocks, planes);
+    auto go = [&](auto kc, auto pc) {
+        constexpr int K = decltype(kc)::value;
+        constexpr bool PREV = decltype(pc)::value;
+        if (out) state_kernel<true, K, PREV><<<g, b, 0, s>>>(N, store_of(l), blocks, planes);
+        else state_kernel<false, K, PREV><<<g, b, 0, s>>>(N, store_of(l), blocks, planes);
+    };
+    using std::integral_constant;
+    if (part == STATE_PREV) {
+        go(integral_constant<int, 5>{}, std::true_type{});
+    } else if (part == STATE_HEAD) {
+        go(integral_constant<int, kStateHead>{}, std::false_type{});
+    } else if (part == STATE_TAIL) {
+        blocks += kStateHead * f32::kBlk;
+        planes += (size_t)kStateHead * N;
+        go(integral_constant<int, 38 - kStateHead>{}, std::false_type{});
     } else {
-        return cudaErrorInvalidValue;
+        go(integral_constant<int, 38>{}, std::false_type{});
     }
     return cudaGetLastError();
 }

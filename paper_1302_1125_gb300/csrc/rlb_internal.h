@@ -112,9 +112,11 @@ cudaError_t launch_sym(int fp32, int expand, int sym, int N, const Layout &l, vo
                        unsigned *status, cudaStream_t s);
 cudaError_t launch_macro(int fp32, int N, const Layout &l, const void *f, const void *h, double *out,
                          unsigned *status, cudaStream_t s, int lat = 0);
-// FP32 blocks <-> compact planes of N: the 38 populations (k = 38) or the 5
-// previous-level values (k = 5) of every cell
-cudaError_t launch_state(bool out, int N, const Layout &l, int k, float *blocks, float *planes, cudaStream_t s);
+// FP32 blocks <-> compact planes of N: the 38 populations of every cell, their
+// first kStateHead or the rest (planes: of all 38), or the 5 previous-level values
+enum StatePart { STATE_ALL, STATE_HEAD, STATE_TAIL, STATE_PREV };
+constexpr int kStateHead = 5;
+cudaError_t launch_state(bool out, int N, const Layout &l, StatePart part, float *blocks, float *planes, cudaStream_t s);
 // partial holds 5 * totals_blocks(N) doubles; out 5 doubles (device)
 int totals_blocks(int N);
 cudaError_t launch_totals(int fp32, int N, const Layout &l, const void *f, const void *h,
