@@ -62,8 +62,8 @@ __device__ __forceinline__ void tube_ends(int nx, int x0, int &ol, int &orr, uns
 // Populations in blocks of 32 cells and stencils straight into registers, as
 // on grids (f32::BlockIO); plain loads, which after the block or cluster
 // barrier see what the other threads of the cluster wrote in the step before.
-// MAXT = launch bound: 512 caps the kernel at 128 registers (some spill),
-// 384 at 168, 256 leaves it unconstrained; the autotuner picks.
+// MAXT = launch bound: 512 caps the kernel at 128 registers, 384 at 168, 256
+// leaves it unconstrained (147; none spills); the autotuner picks.
 template <int MAXT, int NP>
 __global__ void __launch_bounds__(MAXT, 1) tubes_kernel(const Args a)
 {

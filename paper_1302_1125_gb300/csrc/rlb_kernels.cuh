@@ -266,7 +266,8 @@ __device__ __forceinline__ void flag(const StepParams &p, unsigned bits)
 // warps count: at 128 registers (four blocks of 128 per SM; the own
 // populations are loaded again rather than held) the 256 x 128 x 128 cloud
 // takes 6.3 ms a step, with two, three and five blocks 8.6, 6.8 and 6.6 (9.9
-// before, at 255 registers).
+// before, at 255 registers).  At 128 it spills 76 to 140 bytes a thread in 3-D, up
+// to 52 in 2-D.
 #ifndef RLB_F64_MINB
 #define RLB_F64_MINB 4
 #endif

@@ -508,7 +508,8 @@ constexpr int item_at(int s)
 // ahead) took 74 % of the L1 data path's wavefronts: every value went through
 // it three times.  Distance measured on the 512 x 256 x 256 and 2048 x 1024
 // shock-clouds, ms a step at 1 / 2 / 3 / 4 items: 4.29 / 3.78 / 3.55 / 3.97
-// and 0.199 / 0.190 / 0.177 / 0.183 (4 items spill); an L2 prefetch of the
+// and 0.199 / 0.190 / 0.177 / 0.183 (3-D: 92 bytes a thread spilled at 3, none
+// at 2); an L2 prefetch of the
 // rows ahead on top measured slower (3.59 to 3.76 ms, 0.180 to 0.205 ms).
 template <int DIM, bool EULER, int NP, int LAT, bool ODDP>
 struct BlockIO {
@@ -925,8 +926,11 @@ __device__ __forceinline__ void slab_order(int slab_by, unsigned &bx, unsigned &
 #define RLB_F32_BY 8
 #endif
 
-// threads per block of the 1-D form (us for 200 steps with 32 / 64 / 128: 800
-// cells symmetric 815 / 795 / 736, 8192 cells 1362 / 1398 / 1416)
+// threads per block of the 1-D form: one size for all lengths.  us a step with 32 /
+// 64 / 128, all populations (1-D reduction): 200 cells 5.28 / 5.22 / 5.36 (3.12 /
+// 3.17 / 3.21), 800 6.12 / 5.83 / 5.20 (3.61 / 3.46 / 3.22), 2000 6.35 / 6.23 /
+// 5.74, 8192 6.41 / 6.68 / 6.64 (3.72 / 4.12 / 4.07), 20000 6.89 / 6.55 / 6.44,
+// 200000 16.15 / 16.02 / 15.93; where 128 is not the best it loses 3 % (9 %)
 constexpr int kTubeThreads = 128;
 constexpr int kParkH = 11;   // f2 slots per thread in shared memory of the parked h coefficients
 // dynamic shared memory of one block of nthr threads
