@@ -579,7 +579,7 @@ static bool in_one_allocation(const void *p, size_t bytes)
 // only.  2.9 GB to host memory 15.1 ms, one after the other 15.8, a bare copy 15.0.
 static rlb_status copy_blocks(rlb_ctx *ctx, void *buf, bool out)
 {
-    cudaPointerAttributes at;
+    cudaPointerAttributes at{};
     const bool known = cudaPointerGetAttributes(&at, buf) == cudaSuccess;
     if (!known) cudaGetLastError();
     const bool near = known && ((at.type == cudaMemoryTypeDevice && at.device == ctx->device) || at.type == cudaMemoryTypeHost);
