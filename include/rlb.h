@@ -290,7 +290,7 @@ RLB_API const char *rlb_status_string(int status);
  * "fp32_tiles" (tiles of
  * 64 x 8 cells, each thread loading its own stencil into registers), "fp32_linear", "fp32_1d", "fp32_rec64" (recovery_fp64),
  * "fp64_tiles", "fp64_linear", "fp64_small" (grids with fewer than 128 cells
- * per SM, under symmetry_1d up to 80: four warps share 32 cells; in Euler mode
+ * per SM, 80 under symmetry_1d: four warps share 32 cells; in Euler mode
  * blocks of one to four warps), "fp64_1d".  The
  * results are the same whichever kernel runs.  NULL ctx: "none". */
 RLB_API const char *rlb_step_kernel(const rlb_ctx *ctx);
